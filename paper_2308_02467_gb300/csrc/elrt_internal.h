@@ -123,6 +123,12 @@ elrt_status tc_lu_resolve(elrt_ctx* ctx, float* M, int64_t ld, int64_t estride, 
                           int nrhs, bool f16, const double* res_max);
 size_t tc_lu_side_floats(const Tab& t, int64_t ld);
 
+// ---- float-float refinement residual of the common element shapes (residual.cu): mode 0 X = D, mode 1
+// X += D; R = -B^ - A X over D, maxres[e] = max |R|.  X: [n][nu][nin] float-float.
+bool residual_eo_fits(const Tab& t);
+elrt_status residual_eo(elrt_ctx* ctx, double h, const double* h_elem, const double* kappa, const double* omega, float* M,
+                        int64_t ld, int64_t estride, void* X, int mode, double* maxres, int64_t n);
+
 // ---- launchers implemented in global.cu
 elrt_status global_apply(elrt_ctx* ctx, int nx, int nz, const void* A, int dtype, const double* x, double* y);
 elrt_status global_solve(elrt_ctx* ctx, int nx, int nz, const void* A, int dtype, const double* inflow,

@@ -646,7 +646,7 @@ __global__ void __launch_bounds__(kThreads) k_residual(Tab t, double h, const do
 // circulant angular sum of -S X (eq. hdg_local_mat).
 //   mode 0: X = D;  mode 1: X += D;  mode 2: X += D and no residual.
 // In modes 0 and 1, R = -B^ - A X is written over D (FP32) and maxres[e] = max |R|.
-// N1T / NAT fix n1 = p + 1 and N at compile time (0: read from the table).
+// This form takes any p and N; the common shapes have their own kernel in residual.cu.
 // ------------------------------------------------------------------------------------------------
 constexpr int kResThreads = 512;
 
@@ -671,15 +671,14 @@ __device__ __forceinline__ void ld_pair(const ff* p, ff& a, ff& b) {
 
 // XS: type of the staged X chunk: float for mode 0 (half the shared memory, so twice the
 // columns per pass), float-float for modes 1 and 2
-template <int N1T, int NAT, typename XS>
+template <typename XS>
 __global__ void __launch_bounds__(kResThreads, 2) k_residual_ff(Tab t, double h, const double* __restrict__ h_elem,
                                                              const double* __restrict__ kappa,
                                                              const double* __restrict__ omega, float* __restrict__ Mall,
                                                              int64_t ld, int64_t estride, ff* __restrict__ Xall, int mode,
                                                              int CWR, double* __restrict__ maxres, int64_t E) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int n1 = N1T > 0 ? N1T : t.n1;
-    const int N = NAT > 0 ? NAT : t.N;
+    const int n1 = t.n1, N = t.N;
     const int nm = n1 * n1, nu = nm * N, nin = t.nin, p = n1 - 1;
     // shared memory (residual_ff_smem): X chunk, then the per-element tables at their exact sizes
     XS* Xs = reinterpret_cast<XS*>(smem_raw);  // [nu][CWR]
@@ -1212,7 +1211,7 @@ int residual_ff_cwr(const Tab& t, size_t xs) {
     return cwr;
 }
 
-template <int N1T, int NAT, typename XS>
+template <typename XS>
 elrt_status launch_residual_ff(elrt_ctx* ctx, double h, const double* h_elem, const double* kappa, const double* omega,
                                float* M, int64_t ld, int64_t estride, ff* X, int mode, double* maxres, int64_t n) {
     const Tab& t = ctx->tab;
@@ -1220,7 +1219,7 @@ elrt_status launch_residual_ff(elrt_ctx* ctx, double h, const double* h_elem, co
     if (cwr < 2) return ctx_fail(ctx, ELRT_EINVAL, "float-float residual: element too large for two staged columns");
     const size_t smem = residual_ff_smem(t, cwr, sizeof(XS));
     cudaError_t e =
-        cudaFuncSetAttribute(k_residual_ff<N1T, NAT, XS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(k_residual_ff<XS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_check(ctx, e, "smem attribute");
     // a batch too small to fill the GPU spreads each element's column chunks over several blocks
     const int nchunk = (t.nin + cwr - 1) / cwr;
@@ -1230,29 +1229,23 @@ elrt_status launch_residual_ff(elrt_ctx* ctx, double h, const double* h_elem, co
         if (e != cudaSuccess) return cuda_check(ctx, e, "residual maxima");
     }
     ProfScope ps(ctx, "residual", 1, residual_bytes(t, sizeof(float), mode, n), residual_flops(t, mode, n));
-    k_residual_ff<N1T, NAT, XS><<<dim3((unsigned)n, (unsigned)gy), kResThreads, smem, ctx->stream>>>(
+    k_residual_ff<XS><<<dim3((unsigned)n, (unsigned)gy), kResThreads, smem, ctx->stream>>>(
         t, h, h_elem, kappa, omega, M, ld, estride, X, mode, cwr, maxres, n);
     return cuda_check(ctx, cudaGetLastError(), "residual launch");
 }
 
-template <int N1T, int NAT>
-elrt_status launch_residual_mode(elrt_ctx* ctx, double h, const double* h_elem, const double* kappa,
-                                 const double* omega, float* M, int64_t ld, int64_t estride, ff* X, int mode,
-                                 double* maxres, int64_t n) {
-    if (mode == 0)
-        return launch_residual_ff<N1T, NAT, float>(ctx, h, h_elem, kappa, omega, M, ld, estride, X, mode, maxres, n);
-    return launch_residual_ff<N1T, NAT, ff>(ctx, h, h_elem, kappa, omega, M, ld, estride, X, mode, maxres, n);
-}
-
-// unrolled shapes for Q6 elements with 16 or 28 angular cells; any other shape reads the table
+// common element shapes take the split-sum kernel of residual.cu (about half the multiply-adds), any
+// other shape the general kernel above
 elrt_status run_residual_ff(elrt_ctx* ctx, double h, const double* h_elem, const double* kappa, const double* omega,
                             float* M, int64_t ld, int64_t estride, ff* X, int mode, double* maxres, int64_t n) {
     const Tab& t = ctx->tab;
-    if (t.n1 == 7 && t.N == 16)
-        return launch_residual_mode<7, 16>(ctx, h, h_elem, kappa, omega, M, ld, estride, X, mode, maxres, n);
-    if (t.n1 == 7 && t.N == 28)
-        return launch_residual_mode<7, 28>(ctx, h, h_elem, kappa, omega, M, ld, estride, X, mode, maxres, n);
-    return launch_residual_mode<0, 0>(ctx, h, h_elem, kappa, omega, M, ld, estride, X, mode, maxres, n);
+    if (mode != 2 && residual_eo_fits(t)) {
+        ProfScope ps(ctx, "residual", 1, residual_bytes(t, sizeof(float), mode, n), residual_flops(t, mode, n));
+        return residual_eo(ctx, h, h_elem, kappa, omega, M, ld, estride, X, mode, maxres, n);
+    }
+    if (mode == 0)
+        return launch_residual_ff<float>(ctx, h, h_elem, kappa, omega, M, ld, estride, X, mode, maxres, n);
+    return launch_residual_ff<ff>(ctx, h, h_elem, kappa, omega, M, ld, estride, X, mode, maxres, n);
 }
 
 template <typename O>
