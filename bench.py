@@ -918,7 +918,7 @@ def run_ours(args, rank, world, local_rank):
     torch.cuda.synchronize()
     ms_profiled = ev2.elapsed_time(ev3) / args.steps
     names = ("assemble", "lu_factor_solve", "lu_resolve", "lu_tc_diag", "lu_tc_rowcol", "lu_tc_update", "residual",
-             "restrict", "status", "gemv", "krylov", "sweep")
+             "adjoint", "restrict", "status", "gemv", "krylov", "sweep")
     prof = {k: ctx.elrt_profile_get(k) for k in names}
     work = {k: ctx.elrt_profile_work(k) for k in names}
     ctx.elrt_profile_enable(False)

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include <map>
@@ -36,6 +37,13 @@ __host__ __device__ inline int face_node(int F, int m, int p) {
         case 2: return m + n1 * p;
         default: return n1 * m;
     }
+}
+
+// the power of two that brings |v| into [0.5, 1)
+__host__ __device__ inline float unit_scale(double v) {
+    int ex;
+    frexp(v, &ex);
+    return ldexpf(1.f, -ex);
 }
 
 // Launch parameters the autotuner (tune.cpp) measures and sets; the defaults are the hand-chosen ones.
@@ -124,10 +132,17 @@ elrt_status tc_lu_resolve(elrt_ctx* ctx, float* M, int64_t ld, int64_t estride, 
 size_t tc_lu_side_floats(const Tab& t, int64_t ld);
 
 // ---- float-float refinement residual of the common element shapes (residual.cu): mode 0 X = D, mode 1
-// X += D; R = -B^ - A X over D, maxres[e] = max |R|.  X: [n][nu][nin] float-float.
+// X += D; R = -B^ - A X over D, maxres[e] = max |R|.  X: [n][nu][nin] float-float.  Mode 3, for the adjoint
+// correction: every -B^ column scaled by unit_scale of its entry, D left as it is, R to its own buffer
+// [n][nu][nin], and the sums of D over the angular cells [n][nm][nin] to X.
 bool residual_eo_fits(const Tab& t);
 elrt_status residual_eo(elrt_ctx* ctx, double h, const double* h_elem, const double* kappa, const double* omega, float* M,
-                        int64_t ld, int64_t estride, void* X, int mode, double* maxres, int64_t n);
+                        int64_t ld, int64_t estride, void* X, int mode, double* maxres, int64_t n, float* R = nullptr);
+
+// ---- last refinement step by an adjoint product (adjoint.cu)
+bool adjoint_fits(const Tab& t);
+elrt_status adjoint_correct(elrt_ctx* ctx, const float* M, int64_t ld, int64_t estride, const float* R, const void* sum,
+                            float* in2out, float* in2sol, int* err, int64_t n);
 
 // ---- launchers implemented in global.cu
 elrt_status global_apply(elrt_ctx* ctx, int nx, int nz, const void* A, int dtype, const double* x, double* y);

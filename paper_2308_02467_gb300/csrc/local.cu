@@ -114,7 +114,11 @@ __device__ __forceinline__ float aug_entry_f(const Tab& t, const AugF& f, int k,
     return v;
 }
 
-// Grid: (E, N).  Block (e, k) writes rows (k, 0..nm-1) of element e; columns >= nu + nin are 0.
+// Grid: (E, N).  Block (e, k) writes rows (k, 0..nm-1) of element e; columns >= nu + nin are 0, or, with iso
+// (FP32), nm more right-hand sides follow the -B^ columns: the isotropic unit sources, 1 in row (k, i) of
+// column nu + nin + i, and every -B^ column is scaled by the power of two that brings its entry into
+// [0.5, 1) (its solution is then as accurate in the 3xFP16 updates as the largest column's: the entries of
+// grazing directions at end nodes are ~0.01, where FP16 remainders are subnormal).
 // Also validates the inputs (flags[0] |= 1 on a negative or non-finite kappa / h, omega outside [0, 1],
 // or kappa_hat = kappa h / 2 above 1e30, beyond which the FP32 modes would overflow).
 template <typename T>
@@ -122,7 +126,7 @@ __global__ void __launch_bounds__(kThreads) k_assemble(Tab t, double h, const do
                                                        const double* __restrict__ kappa,
                                                        const double* __restrict__ omega, T* __restrict__ M,
                                                        int64_t ld, int64_t estride, T* __restrict__ rhs_out,
-                                                       int64_t rhs_ld, int* flags) {
+                                                       int64_t rhs_ld, int* flags, int iso) {
     __shared__ double kh[ELRT_MAX_N1 * ELRT_MAX_N1];
     const int64_t e = blockIdx.x;
     const int k = blockIdx.y;
@@ -176,6 +180,7 @@ __global__ void __launch_bounds__(kThreads) k_assemble(Tab t, double h, const do
             __syncwarp();
             const int n1 = t.n1, a = i % n1, b = i / n1;
             const int ncand = 1 + 2 * (n1 - 1) + (t.N - 1) + 4;
+            if (iso && lane == 31) row[t.nu + t.nin + i] = T(1);
             for (int q = lane; q < ncand; q += 32) {
                 int c = -1;
                 if (q == 0) {
@@ -203,7 +208,7 @@ __global__ void __launch_bounds__(kThreads) k_assemble(Tab t, double h, const do
                 if (c >= 0) {
                     if constexpr (sizeof(T) == 4) {
                         const float v = aug_entry_f(t, fa, k, i, c);
-                        row[c] = v;
+                        row[c] = iso && c >= t.nu ? v * unit_scale(v) : v;
                         amax = fmaxf(amax, fabsf(v));
                     } else {
                         row[c] = (T)aug_entry(t, k, i, c, kh, om);
@@ -1213,7 +1218,7 @@ elrt_status local_assemble_f64(elrt_ctx* ctx, int64_t E, double h, const double*
         ProfScope ps(ctx, "assemble", 1, (double)n * (8.0 * t.nu * (t.nu + t.nin) + 8.0 * (t.nm + 2)));
         k_assemble<double><<<grid, kThreads, 0, ctx->stream>>>(
             t, h, h_elem ? h_elem + e0 : nullptr, kappa + e0 * t.nm, omega + e0, A + e0 * (int64_t)t.nu * t.nu, t.nu,
-            (int64_t)t.nu * t.nu, rhs + e0 * (int64_t)t.nu * t.nin, t.nin, ctx->d_flags);
+            (int64_t)t.nu * t.nu, rhs + e0 * (int64_t)t.nu * t.nin, t.nin, ctx->d_flags, 0);
     }
     s = cuda_check(ctx, cudaGetLastError(), "k_assemble launch");
     if (s) return s;
@@ -1377,11 +1382,17 @@ elrt_status build_chunked(elrt_ctx* ctx, int64_t E, double h, const double* h_el
                           int32_t* elem_status, elrt_local_stats* stats, const elrt_local_extras* ex) {
     const Tab& t = ctx->tab;
     const bool has_src = ex && ex->source;
-    Tab tl = t;  // the LU's right-hand sides: the -B^ columns, then the source column
-    tl.nrhs = t.nin + (has_src ? 1 : 0);
+    const bool ir = (mode != ELRT_LOCAL_FP64);
+    // one refinement step whose caller wants FP32 in2out / in2sol alone: the correction of the operators by
+    // an adjoint product (adjoint.cu), with the isotropic unit sources as nm more right-hand sides.  A build
+    // with statistics, status words, a source or A_i2u needs the corrected solution itself, and FP64 operators
+    // the re-solve's last digits.
+    const bool adj = sizeof(T) == 4 && ir && steps == 1 && out_dtype == ELRT_F32 && !stats && !elem_status && !has_src && !(ex && ex->in2rad) &&
+                     residual_eo_fits(t) && adjoint_fits(t);
+    Tab tl = t;  // the LU's right-hand sides: the -B^ columns, then the source column or the unit sources
+    tl.nrhs = t.nin + (has_src ? 1 : 0) + (adj ? t.nm : 0);
     const int64_t ld = ((t.nu + tl.nrhs + 31) / 32) * 32;
     const int64_t estride = (int64_t)t.nu * ld;
-    const bool ir = (mode != ELRT_LOCAL_FP64);
     double bmax = 0.0;  // max |B^| entry, the scale of the residuals
     for (int F = 0; F < 4; ++F)
         for (int k = 0; k < t.N; ++k)
@@ -1389,11 +1400,15 @@ elrt_status build_chunked(elrt_ctx* ctx, int64_t E, double h, const double* h_el
     const bool want_res = ir || stats || elem_status;
     const bool tc = (mode == ELRT_LOCAL_TF32_IR);
     const size_t side_per = tc ? tc_lu_side_floats(t, ld) * sizeof(float) : 0;
-    // bytes per element: M, ipiv, status, maxres, the FP64 solution when refining / measuring,
-    // and the split operand buffers of the tensor-core LU
+    // bytes per element: M, ipiv, status, maxres, the float-float or FP64 solution when refining /
+    // measuring (the adjoint step: the residual and the angular sums), and the split operand buffers of the
+    // tensor-core LU
+    const size_t sol_per = adj        ? (size_t)t.nu * t.nin * sizeof(float) + (size_t)t.nm * t.nin * sizeof(double)
+                           : want_res ? (size_t)t.nu * t.nin * sizeof(double)
+                                      : 0;
     const size_t src_per = (has_src && ir) ? (size_t)t.nu * sizeof(double) : 0;  // refined source column
     const size_t per = estride * sizeof(T) + t.nu * sizeof(int) + sizeof(int) + sizeof(double) +
-                       (want_res ? (size_t)t.nu * t.nin * sizeof(double) : 0) + side_per + src_per;
+                       sol_per + side_per + src_per;
     // workspace of one chunk: an eighth of the device memory, at most 32 GB (4096 elements at p = 6,
     // N = 16 on a 288 GB device: one chunk for a 64 x 64 field, half the launches of 16 GB chunks)
     const size_t budget = std::min<size_t>((size_t)32 << 30, ctx->dev_bytes / 8);
@@ -1408,7 +1423,7 @@ elrt_status build_chunked(elrt_ctx* ctx, int64_t E, double h, const double* h_el
     unsigned char* base = (unsigned char*)ctx->ws;
     T* M = (T*)base;
     double* X64 = (double*)(base + (size_t)chunk * estride * sizeof(T));
-    double* maxres = X64 + (want_res ? (size_t)chunk * t.nu * t.nin : 0);
+    double* maxres = (double*)((unsigned char*)X64 + (size_t)chunk * sol_per);
     int* ipiv = (int*)(maxres + chunk);
     int* estat = ipiv + (size_t)chunk * t.nu;
     float* side = tc ? (float*)(((uintptr_t)(estat + chunk) + 255) & ~(uintptr_t)255) : nullptr;
@@ -1432,7 +1447,7 @@ elrt_status build_chunked(elrt_ctx* ctx, int64_t E, double h, const double* h_el
             dim3 grid((unsigned)m, t.N);
             ProfScope ps(ctx, "assemble", 1, (double)m * (sizeof(T) * (double)t.nu * (t.nu + t.nin) + 8.0 * (t.nm + 2)));
             k_assemble<T><<<grid, kThreads, 0, ctx->stream>>>(t, h, he ? he + a0 : nullptr, ka + a0 * t.nm, om + a0,
-                                                              M + a0 * estride, ld, estride, nullptr, 0, ctx->d_flags);
+                                                              M + a0 * estride, ld, estride, nullptr, 0, ctx->d_flags, adj);
         }
         if (has_src)
             k_source_column<T><<<(unsigned)n, kThreads, 0, ctx->stream>>>(t, h, he, ex->source + e0 * t.nu, M, ld,
@@ -1471,7 +1486,18 @@ elrt_status build_chunked(elrt_ctx* ctx, int64_t E, double h, const double* h_el
         };
         void* o_i2o = (unsigned char*)in2out + (size_t)e0 * t.nin * t.nin * osz;
         void* o_i2m = (unsigned char*)in2sol + (size_t)e0 * t.nm * t.nin * osz;
-        if (want_res) {
+        if (adj) {
+            if constexpr (sizeof(T) == 4) {
+                ff* sum = (ff*)X64;  // [n][nm][nin], then the residual [n][nu][nin]
+                float* R = (float*)(sum + (size_t)chunk * t.nm * t.nin);
+                {
+                    ProfScope ps(ctx, "residual", 1, 8.0 * t.nu * t.nin * (double)n + 8.0 * t.nm * t.nin * (double)n,
+                                 residual_flops(t, 0, n));
+                    s = residual_eo(ctx, h, he, ka, om, M, ld, estride, sum, 3, nullptr, n, R);
+                }
+                if (!s) s = adjoint_correct(ctx, M, ld, estride, R, sum, (float*)o_i2o, (float*)o_i2m, ctx->d_flags + 2, n);
+            }
+        } else if (want_res) {
             if constexpr (sizeof(T) == 4)
                 s = run_residual_ff(ctx, h, he, ka, om, M, ld, estride, (ff*)X64, 0, maxres, n);
             else
@@ -1565,6 +1591,7 @@ elrt_status build_chunked(elrt_ctx* ctx, int64_t E, double h, const double* h_el
             s = cuda_check(ctx, cudaGetLastError(), "source restriction launch");
             if (s) return s;
         }
+        if (!stats && !elem_status) continue;  // nobody reads them
         ProfScope ps(ctx, "status", elem_status ? 2 : 1);
         k_reduce_status<<<(unsigned)((n + 255) / 256), 256, 0, ctx->stream>>>(
             estat, want_res ? maxres : nullptr, n, ctx->d_flags + 1, (unsigned long long*)(ctx->d_flags + 4));
@@ -1679,7 +1706,7 @@ elrt_status static_build(const Tab& t, cudaStream_t sm, unsigned char* scratch, 
         const double* ka = kappa + e0 * t.nm;
         const double* om = omega + e0;
         if (cudaMemsetAsync(estat, 0, n * sizeof(int), sm) != cudaSuccess) return ELRT_ECUDA;
-        k_assemble<T><<<dim3((unsigned)n, t.N), kThreads, 0, sm>>>(t, h, he, ka, om, M, ld, estride, nullptr, 0, flags);
+        k_assemble<T><<<dim3((unsigned)n, t.N), kThreads, 0, sm>>>(t, h, he, ka, om, M, ld, estride, nullptr, 0, flags, 0);
         if (lu_run<T, NB, QN>(t, sm, M, ld, estride, ipiv, estat, n, false)) return ELRT_ECUDA;
         void* o_i2o = (unsigned char*)in2out + (size_t)e0 * t.nin * t.nin * osz;
         void* o_i2m = (unsigned char*)in2sol + (size_t)e0 * t.nm * t.nin * osz;

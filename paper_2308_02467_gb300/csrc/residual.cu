@@ -129,12 +129,16 @@ struct ResCfg {
 };
 
 // mode 0: X = D (XS float);  mode 1: X += D (XS ff).  R over D, maxres[e] = max |R|.
-template <int N1, int N, typename XS>
+// ADJ (XS float, for the adjoint correction of adjoint.cu): the columns of B^ carry the power-of-two scales of
+// the assembly (unit_scale of their entry), X = D stays where it is, R goes to Rall
+// [E][NU][nin], Xall takes the sums of X over the angular cells [E][NM][nin] instead of X, and no maximum is
+// formed.
+template <int N1, int N, typename XS, bool ADJ>
 __global__ void __launch_bounds__(ResCfg<N1, N, XS>::T, ResCfg<N1, N, XS>::BLOCKS)
     k_residual_eo(const __grid_constant__ Tab t, const __grid_constant__ ResTab rt, double h,
                   const double* __restrict__ h_elem, const double* __restrict__ kappa, const double* __restrict__ omega,
                   float* __restrict__ Mall, int64_t ld, int64_t estride, ff* __restrict__ Xall,
-                  double* __restrict__ maxres) {
+                  double* __restrict__ maxres, float* __restrict__ Rall) {
     using Cfg = ResCfg<N1, N, XS>;
     constexpr int NM = Cfg::NM, NU = Cfg::NU, T = Cfg::T, P = N1 - 1, G = T / kCW;
     constexpr bool F = Cfg::F;
@@ -149,7 +153,9 @@ __global__ void __launch_bounds__(ResCfg<N1, N, XS>::T, ResCfg<N1, N, XS>::BLOCK
     const int nin = t.nin, tid = threadIdx.x;
     const int64_t e = blockIdx.x;
     float* M = Mall + e * estride + NU;  // the right-hand-side columns
-    ff* X = Xall + e * (int64_t)NU * nin;
+    ff* X = Xall + e * (int64_t)(ADJ ? NM : NU) * nin;
+    float* Rp = ADJ ? Rall + e * (int64_t)NU * nin : M;
+    const int64_t rld = ADJ ? nin : ld;
     const int step = gridDim.y * kCW;
     auto prefetch = [&](int cs, XS* dst) {  // first pass: the chunk's columns of D (two 16-byte halves a row)
         if constexpr (F) {
@@ -188,7 +194,8 @@ __global__ void __launch_bounds__(ResCfg<N1, N, XS>::T, ResCfg<N1, N, XS>::BLOCK
             __syncthreads();  // the chunk has landed; the last pass over the other buffer is done
             xs = Xs + (size_t)buf * NU * kCW;
             if (cs + step < nin) prefetch(cs + step, Xs + (size_t)(buf ^ 1) * NU * kCW);
-            for (int r = g; r < NU; r += G) X[(int64_t)r * nin + cs + col] = ff{xs[r * kCW + col], 0.f};
+            if constexpr (!ADJ)
+                for (int r = g; r < NU; r += G) X[(int64_t)r * nin + cs + col] = ff{xs[r * kCW + col], 0.f};
         } else {
             __syncthreads();
             constexpr int SB = 8;  // independent loads in flight
@@ -220,6 +227,12 @@ __global__ void __launch_bounds__(ResCfg<N1, N, XS>::T, ResCfg<N1, N, XS>::BLOCK
             XS x[N];
 #pragma unroll
             for (int l = 0; l < N; ++l) x[l] = xs[(l * NM + i) * kCW + col];
+            if constexpr (ADJ) {
+                ff m = sum2(x[0], x[1]);
+#pragma unroll
+                for (int l = 2; l < N; ++l) m = ff_add(m, ff{x[l], 0.f});
+                X[(int64_t)i * nin + cs + col] = m;
+            }
             const ff sc = scoef[i];
             angular<N>(rt, x, [&](int k, ff y) {
                 ff acc = mul0(dcoef[k * NM + i], x[k]);
@@ -246,7 +259,12 @@ __global__ void __launch_bounds__(ResCfg<N1, N, XS>::T, ResCfg<N1, N, XS>::BLOCK
         const int c = cs + col, Fc = c / t.nface, rem = c - Fc * t.nface, m = rem / t.half;
         const int kin = t.inc[Fc][rem - m * t.half];
         const int tr = kin * NM + face_node(Fc, m, P);
-        const ff tv = ff_from_double(-t.w[m] * t.sdn[Fc][kin]);
+        ff tv = ff_from_double(-t.w[m] * t.sdn[Fc][kin]);
+        if constexpr (ADJ) {
+            // the scale the assembly used: the power of two is that of the entry in FP32 arithmetic
+            const float us = unit_scale((float)-t.w[m] * (float)t.sdn[Fc][kin]);
+            tv = ff{tv.h * us, tv.l * us};
+        }
         for (int q = g; q < N * N1; q += G) {
             const int k = q / N1, a = q - k * N1, r0 = k * NM + a;
             XS x[N1];
@@ -260,11 +278,12 @@ __global__ void __launch_bounds__(ResCfg<N1, N, XS>::T, ResCfg<N1, N, XS>::BLOCK
                 acc = ff_norm(acc.h, acc.l);
                 const ff res = r == tr ? ff_add(tv, neg(acc)) : neg(acc);
                 const float rf = __fadd_rn(res.h, res.l);
-                rmax = fmaxf(rmax, fabsf(rf));
-                M[(int64_t)r * ld + c] = rf;
+                if constexpr (!ADJ) rmax = fmaxf(rmax, fabsf(rf));
+                Rp[(int64_t)r * rld + c] = rf;
             });
         }
     }
+    if constexpr (ADJ) return;
     for (int off = 16; off > 0; off >>= 1) rmax = fmaxf(rmax, __shfl_down_sync(0xffffffffu, rmax, off));
     if ((tid & 31) == 0) red[tid >> 5] = rmax;
     __syncthreads();
@@ -304,29 +323,31 @@ struct Args {
     int64_t ld, estride;
     ff* X;
     double* maxres;
+    float* R;
     int64_t n;
 };
 
-template <int N1, int N, typename XS>
+template <int N1, int N, typename XS, bool ADJ = false>
 elrt_status launch(const Args& a) {
     using Cfg = ResCfg<N1, N, XS>;
     const Tab& t = a.ctx->tab;
-    cudaError_t e = cudaFuncSetAttribute(k_residual_eo<N1, N, XS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
+    cudaError_t e = cudaFuncSetAttribute(k_residual_eo<N1, N, XS, ADJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
     if (e != cudaSuccess) return cuda_check(a.ctx, e, "smem attribute");
     // a batch too small to fill the GPU spreads each element's column chunks over several blocks
     const int64_t fit = (int64_t)Cfg::BLOCKS * a.ctx->sms / std::max<int64_t>(a.n, 1);
     const int gy = (int)std::max<int64_t>(1, std::min<int64_t>(t.nin / kCW, fit));
-    if (gy > 1) {
+    if (gy > 1 && !ADJ) {
         e = cudaMemsetAsync(a.maxres, 0, (size_t)a.n * sizeof(double), a.ctx->stream);
         if (e != cudaSuccess) return cuda_check(a.ctx, e, "residual maxima");
     }
-    k_residual_eo<N1, N, XS><<<dim3((unsigned)a.n, (unsigned)gy), Cfg::T, Cfg::SMEM, a.ctx->stream>>>(
-        t, make_tab(t), a.h, a.h_elem, a.kappa, a.omega, a.M, a.ld, a.estride, a.X, a.maxres);
+    k_residual_eo<N1, N, XS, ADJ><<<dim3((unsigned)a.n, (unsigned)gy), Cfg::T, Cfg::SMEM, a.ctx->stream>>>(
+        t, make_tab(t), a.h, a.h_elem, a.kappa, a.omega, a.M, a.ld, a.estride, a.X, a.maxres, a.R);
     return cuda_check(a.ctx, cudaGetLastError(), "residual launch");
 }
 
 template <int N1, int N>
 elrt_status launch_mode(const Args& a, int mode) {
+    if (mode == 3) return launch<N1, N, float, true>(a);
     return mode == 0 ? launch<N1, N, float>(a) : launch<N1, N, ff>(a);
 }
 
@@ -340,8 +361,8 @@ bool residual_eo_fits(const Tab& t) {
 }
 
 elrt_status residual_eo(elrt_ctx* ctx, double h, const double* h_elem, const double* kappa, const double* omega, float* M,
-                        int64_t ld, int64_t estride, void* X, int mode, double* maxres, int64_t n) {
-    const Args a{ctx, h, h_elem, kappa, omega, M, ld, estride, (ff*)X, maxres, n};
+                        int64_t ld, int64_t estride, void* X, int mode, double* maxres, int64_t n, float* R) {
+    const Args a{ctx, h, h_elem, kappa, omega, M, ld, estride, (ff*)X, maxres, R, n};
     switch (ctx->tab.n1 * 100 + ctx->tab.N) {
         case 308: return launch_mode<3, 8>(a, mode);
         case 312: return launch_mode<3, 12>(a, mode);
