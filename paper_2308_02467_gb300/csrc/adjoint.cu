@@ -26,11 +26,11 @@
 // with the summation index outermost, so sixteen warps load them with 16-byte loads (four rows of four
 // columns a lane), transpose in registers and write K-major, 128-byte-swizzled tiles of 32 rows of the sum,
 // eight lanes on one row's eight chunks (no bank conflicts); one thread of a seventeenth warp issues the MMAs.
-// Bound by its loads (about 1.9 MB per element in two column tiles, the second tile's from L2); the tensor
-// pipe needs about two thirds of that time.  The epilogue reads X at the outflow rows, adds the correction
+// Bound by the latency of its loads (about 2.4 MB per element in two column tiles, the second tile's mostly
+// from L2; DRAM 25 % and the tensor pipe 28 % busy): 16 warps and two stages of 106 KB are what one SM holds.  The epilogue reads X at the outflow rows, adds the correction
 // and rounds once.  Measured, builds with one refinement step: 4096 elements at p = 6, N = 16, 61.9 -> 51.6 ms
-// (the re-solve and the float-float restriction gone, k_adjoint 5.0 ms, the 49 columns 2 ms); nine elements
-// 1.92 -> 1.29 ms (141 -> 90 launches).
+// (the re-solve and the float-float restriction gone, k_adjoint 4.4 ms, the 49 columns 2 ms), 50.8 ms with its
+// loads as below; nine elements 1.92 -> 1.28 ms (141 -> 90 launches).
 #include <algorithm>
 
 #include "elrt_internal.h"
@@ -39,8 +39,8 @@
 
 namespace {
 
-constexpr int kAdjWarps = 16;                      // operand and epilogue warps
-constexpr int kAdjThreads = 32 * (kAdjWarps + 1);  // and the MMA warp
+constexpr int kAdjWarps = 15;                      // operand warps
+constexpr int kAdjThreads = 32 * (kAdjWarps + 1);  // and the MMA warp; all sixteen run the epilogue
 constexpr int kAdjK = 32;                          // rows of the sum per stage: 128 bytes of FP32
 constexpr int kAdjSmem = 220 * 1024;
 
@@ -67,6 +67,9 @@ __device__ __forceinline__ void mma_tf32_ss(uint32_t d_tmem, uint64_t a_desc, ui
             d_tmem),
         "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate));
 }
+
+// column of operand row w within blocks of 16
+__host__ __device__ constexpr int unperm16(int w) { return (w & ~15) | (4 * (w & 3) + ((w >> 2) & 3)); }
 
 __global__ void __launch_bounds__(kAdjThreads, 1)
     k_adjoint(const __grid_constant__ Tab t, const __grid_constant__ AdjArgs g, float* __restrict__ in2out,
@@ -123,29 +126,34 @@ __global__ void __launch_bounds__(kAdjThreads, 1)
     bool ok = true;
     if (warp < kAdjWarps) {
         // operand tasks of a chunk: 16 columns each, the jw columns of r first, then the nc of XZ; lane: rows
-        // 4 kc .. 4 kc + 3 of the chunk, columns 4 c4 .. 4 c4 + 3 of the task
-        const int kc = lane & 7, c4 = lane >> 3;
-        const int ja = g.jw / 16, ntask = ja + NC / 16;
+        // 4 kc .. 4 kc + 3 of the chunk, columns 4 c4 .. 4 c4 + 3 of the task.  Four neighbouring lanes read 64
+        // bytes of a row (eight rows to eight neighbouring lanes cost four times the L1 wavefronts: k_adjoint
+        // 4.8 against 4.4 ms for 4096 elements); with kc and kc + 4 in a quarter warp and column 4 c4 + q in
+        // operand row 4 q + c4 of its block of 16 (unperm16), the stores of a quarter touch every bank once.
+        const int kc = (lane >> 3) + (lane & 4), c4 = lane & 3;
+        const int ja = g.jw / 16, ntask = ja + NC / 16, half = nu / 2, ld = (int)g.ld;
+        int swz[4];  // byte offset of this lane's chunk for its column q, within the task's 16 rows
+#pragma unroll
+        for (int q = 0; q < 4; ++q) swz[q] = (4 * q + c4) * 128 + ((kc ^ ((4 * q + c4) & 7)) << 4);
         auto load = [&](int task, int k0, float4 (&v)[4]) {
             const bool isr = task < ja;
             const int col = 16 * (isr ? task : task - ja) + 4 * c4;
             const bool in = isr ? j0 + col < nin : col < nin + nm;
+            const float* p = isr ? Re + j0 + col : Me + col;
+            const int rld = isr ? nin : ld;
+            const int k = k0 + 4 * kc;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const int k = k0 + 4 * kc + q;
                 v[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (in && k < nu) {
-                    const int rev = k < nu / 2 ? k + nu / 2 : k - nu / 2;  // the reversed direction's row
-                    v[q] = isr ? __ldcs(reinterpret_cast<const float4*>(Re + (int64_t)k * nin + j0 + col))
-                               : __ldg(reinterpret_cast<const float4*>(Me + (int64_t)rev * g.ld + col));
-                }
+                // XZ: the reversed direction's row
+                const int row = isr ? k + q : (k + q < half ? k + q + half : k + q - half);
+                if (in && k + q < nu) v[q] = __ldg(reinterpret_cast<const float4*>(p + row * rld));
             }
         };
         auto store = [&](unsigned char* st, int task, const float4 (&v)[4]) {
             const bool isr = task < ja;
-            unsigned char* hi = st + (isr ? 0 : 2 * a_bytes);
+            unsigned char* hi = st + (isr ? task * 2048 : 2 * a_bytes + (task - ja) * 2048);  // 16 rows a task
             const int lo = isr ? a_bytes : b_bytes;
-            const int row0 = 16 * (isr ? task : task - ja) + 4 * c4;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 float4 x;
@@ -154,58 +162,111 @@ __global__ void __launch_bounds__(kAdjThreads, 1)
                 if (q == 2) x = make_float4(v[0].z, v[1].z, v[2].z, v[3].z);
                 if (q == 3) x = make_float4(v[0].w, v[1].w, v[2].w, v[3].w);
                 auto low = [](float f) { return f - __uint_as_float(__float_as_uint(f) & 0xFFFFE000u); };
-                unsigned char* p = hi + (row0 + q) * 128 + ((kc ^ ((row0 + q) & 7)) << 4);
-                *reinterpret_cast<float4*>(p) = x;
-                *reinterpret_cast<float4*>(p + lo) = make_float4(low(x.x), low(x.y), low(x.z), low(x.w));
+                *reinterpret_cast<float4*>(hi + swz[q]) = x;
+                *reinterpret_cast<float4*>(hi + swz[q] + lo) = make_float4(low(x.x), low(x.y), low(x.z), low(x.w));
             }
         };
-        for (int ch = 0; ch < nch && ok; ++ch) {
+        // the next chunk's first two tasks are loaded before this chunk's are stored, so their latency passes
+        // behind the wait for the stage, the stores and the MMAs (5.0 -> 4.8 ms)
+        auto load2 = [&](int ch, float4 (&v)[2][4]) {
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+                if (ch < nch && warp + u * kAdjWarps < ntask) load(warp + u * kAdjWarps, ch * kAdjK, v[u]);
+        };
+        auto chunk = [&](int ch, const float4 (&v)[2][4], float4 (&next)[2][4]) {
             const int s = ch % NS;
             unsigned char* st = base + s * stage;
-            bool waited = false;
-            auto wait = [&]() {  // the stage is free (a warp without a task waits too: one arrival per phase)
-                if (!waited) ok = __all_sync(0xffffffffu, tc::mbar_wait(&empty[s], ((ch / NS) & 1) ^ 1, abort) && !*abort);
-                waited = true;
-            };
-            for (int task = warp; task < ntask && ok; task += 2 * kAdjWarps) {  // two tasks' loads in flight
-                float4 v0[4], v1[4];
-                const int t1 = task + kAdjWarps;
-                load(task, ch * kAdjK, v0);
-                if (t1 < ntask) load(t1, ch * kAdjK, v1);
-                wait();
-                if (!ok) break;
-                store(st, task, v0);
-                if (t1 < ntask) store(st, t1, v1);
+            load2(ch + 1, next);
+            // the stage is free (a warp without a task waits too: one arrival per phase)
+            ok = __all_sync(0xffffffffu, tc::mbar_wait(&empty[s], ((ch / NS) & 1) ^ 1, abort) && !*abort);
+            if (!ok) return;
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+                if (warp + u * kAdjWarps < ntask) store(st, warp + u * kAdjWarps, v[u]);
+            for (int task = warp + 2 * kAdjWarps; task < ntask; task += kAdjWarps) {  // (wide elements)
+                float4 w[4];
+                load(task, ch * kAdjK, w);
+                store(st, task, w);
             }
-            wait();
-            if (!ok) break;
             tc::fence_proxy_async();  // written through the generic proxy, read by the MMAs (async proxy)
             __syncwarp();
             if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(&full[s])) : "memory");
+        };
+        float4 va[2][4], vb[2][4];
+        load2(0, va);
+        for (int ch = 0; ch < nch && ok; ch += 2) {
+            chunk(ch, va, vb);
+            if (ok && ch + 1 < nch) chunk(ch + 1, vb, va);
         }
-        // epilogue: lane j of the accumulator, 16 columns at a time, four warps per lane quarter
-        const int quad = warp & 3, jl = 32 * quad + lane, j = j0 + jl;
+    } else {
+        if (lane == 0) {
+            const int n0 = min(NC, 256), n1 = NC - n0;
+            const uint32_t id0 = adj_idesc(n0), id1 = adj_idesc(n1);
+            uint32_t acc = 0;
+            int done = 0;
+            for (int ch = 0; ch < nch; ++ch) {
+                const int s = ch % NS;
+                if (!tc::mbar_wait(&full[s], (ch / NS) & 1, abort)) {
+                    ok = false;
+                    break;
+                }
+                tc::tc_fence_after();
+                const uint32_t st = tc::smem_u32(base + s * stage);
+                const uint64_t ah = tc::sw128_desc(st), al = tc::sw128_desc(st + a_bytes);
+                const uint64_t bh = tc::sw128_desc(st + 2 * a_bytes), bl = tc::sw128_desc(st + 2 * a_bytes + b_bytes);
+                const uint64_t b1 = 256 * 128 / 16;  // the columns from 256 on
+#pragma unroll
+                for (int k = 0; k < kAdjK / 8; ++k) {  // K = 8 per instruction: 32 bytes
+                    mma_tf32_ss(tmem, ah + 2 * k, bh + 2 * k, id0, acc);
+                    if (n1) mma_tf32_ss(tmem + 256, ah + 2 * k, bh + b1 + 2 * k, id1, acc);
+                    acc = 1;
+                    mma_tf32_ss(tmem, al + 2 * k, bh + 2 * k, id0, 1);
+                    if (n1) mma_tf32_ss(tmem + 256, al + 2 * k, bh + b1 + 2 * k, id1, 1);
+                    mma_tf32_ss(tmem, ah + 2 * k, bl + 2 * k, id0, 1);
+                    if (n1) mma_tf32_ss(tmem + 256, ah + 2 * k, bl + b1 + 2 * k, id1, 1);
+                }
+                tc::mma_commit(&empty[s]);
+                ++done;
+            }
+            if (!ok) {
+                atomicOr(g.err, 8192);
+                *abort = 1;
+            }
+            tc::mma_commit(&acc_full);
+            // every MMA has completed before the tensor memory and the barriers go (bounded)
+            const long long t0 = clock64();
+            while (!tc::mbar_try_wait(&acc_full, 0) && clock64() - t0 < tc::kWaitCycles) {
+            }
+            for (int ch = max(0, done - NS); ch < done; ++ch)
+                while (!tc::mbar_try_wait(&empty[ch % NS], (ch / NS) & 1) && clock64() - t0 < tc::kWaitCycles) {
+                }
+        }
+        __syncwarp();
+    }
+    // epilogue: lane j of the accumulator, 16 columns at a time, four warps per lane quarter
+    {
+        const int quad = warp & 3, jl = 32 * quad + unperm16(lane), j = j0 + jl;
         const bool jin = jl < g.jw && j < nin;
-        if (ok) ok = __all_sync(0xffffffffu, tc::mbar_wait(&acc_full, 0, abort) && !*abort);
+        ok = __all_sync(0xffffffffu, ok && tc::mbar_wait(&acc_full, 0, abort) && !*abort);
         if (ok) {
             tc::tc_fence_after();
             const float uj = jin ? us[j] : 1.f;
             const ff* se = g.sum + e * (int64_t)nm * nin;
             float* oo = in2out + e * (int64_t)nin * nin;
             float* om = in2sol + e * (int64_t)nm * nin;
-            for (int b = warp >> 2; b < NC / 16; b += kAdjWarps / 4) {
+            for (int b = warp >> 2; b < NC / 16; b += 4) {
                 float x[16], d[16];
                 const int cb = 16 * b;
 #pragma unroll
                 for (int q = 0; q < 16; ++q) {
-                    const int c = cb + q;
+                    const int c = cb + unperm16(q);
                     x[q] = (jin && c < nin) ? Me[(int64_t)xrow[c] * g.ld + j] : 0.f;
                 }
                 tc::tmem_ld16(tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)cb, d);
                 if (jin) {
 #pragma unroll
                     for (int q = 0; q < 16; ++q) {
-                        const int c = cb + q;
+                        const int c = cb + unperm16(q);
                         if (c < nin) {
                             oo[(int64_t)orow[c] * nin + j] = __fadd_rn(x[q] * uj, d[q] * (scale[c] * uj));
                         } else if (c < nin + nm) {
@@ -221,47 +282,6 @@ __global__ void __launch_bounds__(kAdjThreads, 1)
             atomicOr(g.err, 4096);
             *abort = 1;
         }
-    } else if (lane == 0) {
-        const int n0 = min(NC, 256), n1 = NC - n0;
-        const uint32_t id0 = adj_idesc(n0), id1 = adj_idesc(n1);
-        uint32_t acc = 0;
-        int done = 0;
-        for (int ch = 0; ch < nch; ++ch) {
-            const int s = ch % NS;
-            if (!tc::mbar_wait(&full[s], (ch / NS) & 1, abort)) {
-                ok = false;
-                break;
-            }
-            tc::tc_fence_after();
-            const uint32_t st = tc::smem_u32(base + s * stage);
-            const uint64_t ah = tc::sw128_desc(st), al = tc::sw128_desc(st + a_bytes);
-            const uint64_t bh = tc::sw128_desc(st + 2 * a_bytes), bl = tc::sw128_desc(st + 2 * a_bytes + b_bytes);
-            const uint64_t b1 = 256 * 128 / 16;  // the columns from 256 on
-#pragma unroll
-            for (int k = 0; k < kAdjK / 8; ++k) {  // K = 8 per instruction: 32 bytes
-                mma_tf32_ss(tmem, ah + 2 * k, bh + 2 * k, id0, acc);
-                if (n1) mma_tf32_ss(tmem + 256, ah + 2 * k, bh + b1 + 2 * k, id1, acc);
-                acc = 1;
-                mma_tf32_ss(tmem, al + 2 * k, bh + 2 * k, id0, 1);
-                if (n1) mma_tf32_ss(tmem + 256, al + 2 * k, bh + b1 + 2 * k, id1, 1);
-                mma_tf32_ss(tmem, ah + 2 * k, bl + 2 * k, id0, 1);
-                if (n1) mma_tf32_ss(tmem + 256, ah + 2 * k, bl + b1 + 2 * k, id1, 1);
-            }
-            tc::mma_commit(&empty[s]);
-            ++done;
-        }
-        tc::mma_commit(&acc_full);
-        if (!ok) {
-            atomicOr(g.err, 8192);
-            *abort = 1;
-        }
-        // every MMA has completed before the tensor memory and the barriers go (bounded)
-        const long long t0 = clock64();
-        while (!tc::mbar_try_wait(&acc_full, 0) && clock64() - t0 < tc::kWaitCycles) {
-        }
-        for (int ch = max(0, done - NS); ch < done; ++ch)
-            while (!tc::mbar_try_wait(&empty[ch % NS], (ch / NS) & 1) && clock64() - t0 < tc::kWaitCycles) {
-            }
     }
     tc::tc_fence_before();
     __syncthreads();
