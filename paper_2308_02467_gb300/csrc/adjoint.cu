@@ -317,7 +317,7 @@ elrt_status adjoint_correct(elrt_ctx* ctx, const float* M, int64_t ld, int64_t e
     g.stages = 2 * stage <= kAdjSmem - 1024 ? 2 : 1;
     g.err = err;
     const int smem = g.stages * stage + 1024;
-    cudaError_t e = cudaFuncSetAttribute(k_adjoint, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem(k_adjoint);
     if (e != cudaSuccess) return cuda_check(ctx, e, "smem attribute");
     ProfScope ps(ctx, "adjoint", 1,
                  (double)n * (t.nu * (2.0 * t.nin + t.nm) * 4.0 + t.nm * t.nin * 8.0 + (double)(t.nin + t.nm) * t.nin * 4.0),

@@ -105,6 +105,14 @@ void prof_flush(elrt_ctx* ctx);  // call after a stream synchronisation
 void tune_load(elrt_ctx* ctx);
 
 // ---- host helpers implemented in host.cpp
+// Lets kernel f take all the dynamic shared memory a block can have.  The value is the kernel's own, not a
+// launch's: host threads with contexts of different discretisations launch the same kernels, and one thread's
+// smaller value would make another's launch fail.
+cudaError_t allow_smem(const void* f);
+template <typename F>
+cudaError_t allow_smem(F* f) {
+    return allow_smem((const void*)f);
+}
 bool elrt_disc_valid(const elrt_disc* d);
 bool elrt_fill_tab(const elrt_disc* d, Tab* t);
 elrt_status ctx_fail(elrt_ctx* ctx, elrt_status s, const std::string& msg);

@@ -1383,7 +1383,7 @@ cudaError_t launch_stream(elrt_ctx* ctx, unsigned grid, size_t smem, int nx, int
                           const V* x, const double* g, const V* xself, int alpha, int beta, V* y, const GmState* st,
                           const ArnFuse& fz) {
     const Tab& t = ctx->tab;
-    cudaError_t ce = cudaFuncSetAttribute(k_gemv_stream<V, RPW, AT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t ce = allow_smem(k_gemv_stream<V, RPW, AT>);
     if (ce != cudaSuccess) return ce;
     k_gemv_stream<V, RPW, AT><<<grid, kGvThreads, smem, ctx->stream>>>(nx, nz, t.nin, t.nface, rows, Aop, x, g, xself,
                                                                      alpha, beta, y, st, ctx->d_flags + kGemvFlag, fz);

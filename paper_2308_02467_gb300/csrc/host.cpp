@@ -193,6 +193,13 @@ elrt_status ctx_fail(elrt_ctx* ctx, elrt_status s, const std::string& msg) {
     return s;
 }
 
+cudaError_t allow_smem(const void* f) {
+    cudaFuncAttributes a;
+    cudaError_t e = cudaFuncGetAttributes(&a, f);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - (int)a.sharedSizeBytes);
+}
+
 elrt_status cuda_check(elrt_ctx* ctx, cudaError_t e, const char* what) {
     if (e == cudaSuccess) return ELRT_OK;
     return ctx_fail(ctx, e == cudaErrorMemoryAllocation ? ELRT_ENOMEM : ELRT_ECUDA,

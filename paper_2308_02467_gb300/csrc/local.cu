@@ -1262,10 +1262,10 @@ cudaError_t lu_launch(const Tab& t, cudaStream_t st, T* M, int64_t ld, int64_t e
     const int smem = (int)lu_smem_bytes<T, NB, QN>(t.nu);
     cudaError_t e;
     if (resolve) {
-        e = cudaFuncSetAttribute(k_lu_resolve<T, NB, QN, TH>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        e = allow_smem(k_lu_resolve<T, NB, QN, TH>);
         if (e == cudaSuccess) k_lu_resolve<T, NB, QN, TH><<<(unsigned)n, TH, smem, st>>>(t, M, ld, estride, ipiv, n);
     } else {
-        e = cudaFuncSetAttribute(k_lu_factor_solve<T, NB, QN, TH>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        e = allow_smem(k_lu_factor_solve<T, NB, QN, TH>);
         if (e == cudaSuccess)
             k_lu_factor_solve<T, NB, QN, TH><<<(unsigned)n, TH, smem, st>>>(t, M, ld, estride, ipiv, estat, n);
     }
@@ -1299,7 +1299,7 @@ elrt_status run_residual(elrt_ctx* ctx, double h, const double* h_elem, const do
     int cwr = 32;
     while (cwr > 1 && (size_t)t.nu * (cwr + 1) * sizeof(double) > 212 * 1024) cwr >>= 1;
     const size_t smem = (size_t)t.nu * (cwr + 1) * sizeof(double);
-    cudaError_t e = cudaFuncSetAttribute(k_residual<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_residual<T>);
     if (e != cudaSuccess) return cuda_check(ctx, e, "smem attribute");
     ProfScope ps(ctx, "residual", 1, residual_bytes(t, sizeof(T), mode, n), residual_flops(t, mode, n));
     k_residual<T><<<(unsigned)n, kThreads, smem, ctx->stream>>>(t, h, h_elem, kappa, omega, M, ld, estride, X64, mode,
@@ -1328,7 +1328,7 @@ elrt_status launch_residual_ff(elrt_ctx* ctx, double h, const double* h_elem, co
     if (cwr < 2) return ctx_fail(ctx, ELRT_EINVAL, "float-float residual: element too large for two staged columns");
     const size_t smem = residual_ff_smem(t, cwr, sizeof(XS));
     cudaError_t e =
-        cudaFuncSetAttribute(k_residual_ff<XS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem(k_residual_ff<XS>);
     if (e != cudaSuccess) return cuda_check(ctx, e, "smem attribute");
     // a batch too small to fill the GPU spreads each element's column chunks over several blocks
     const int nchunk = (t.nin + cwr - 1) / cwr;
@@ -1696,7 +1696,7 @@ elrt_status static_build(const Tab& t, cudaStream_t sm, unsigned char* scratch, 
     double* maxres = X64 + (ir ? (size_t)chunk * t.nu * t.nin : 0);
     int* ipiv = (int*)(maxres + chunk);
     int* estat = ipiv + (size_t)chunk * t.nu;
-    if (cudaFuncSetAttribute(k_residual<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)res_smem))
+    if (allow_smem(k_residual<T>))
         return ELRT_ECUDA;
     if (cudaMemsetAsync(flags, 0, 2 * sizeof(int), sm) != cudaSuccess) return ELRT_ECUDA;
     const size_t osz = out_dtype == ELRT_F32 ? sizeof(float) : sizeof(double);

@@ -301,12 +301,8 @@ __global__ void __launch_bounds__(kSwThreads, 1) k_sweep(SweepArgs a, const AT* 
 template <typename AT, int NP>
 cudaError_t launch_sweep(cudaLaunchConfig_t cfg, const SweepArgs& a, const void* A) {
     const size_t smem = (size_t)a.stages * a.nface * 2 * a.nin * sizeof(AT) + (((a.nin + 3) & ~3) + 32) * sizeof(float);
-    static size_t attr = 0;
-    if (smem > attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_sweep<AT, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr = smem;
-    }
+    cudaError_t e = allow_smem(k_sweep<AT, NP>);
+    if (e != cudaSuccess) return e;
     cfg.dynamicSmemBytes = smem;
     return cudaLaunchKernelEx(&cfg, k_sweep<AT, NP>, a, (const AT*)A);
 }
