@@ -395,7 +395,8 @@ elrt_status elrt_solve_batch(elrt_ctx* const* ctxs, int32_t n_ctx, const elrt_fi
  *                eighth of the device memory, at most 32 GB);
  *   lu_pairs     tensor-core LU schedule: 1 = panels in pairs, the second factored after a rank-64
  *                update of its rows and columns, the rest of the matrix updated by both with one
- *                rank-128 tensor-core update; 0 = panels one at a time with rank-64 updates;
+ *                rank-128 tensor-core update (3xFP16 products: two pairs at a time with one
+ *                rank-256 update); 0 = panels one at a time with rank-64 updates;
  *   restart      GMRES restart length of solve calls that pass restart = 0 (default 12).
  * elrt_autotune builds the local operators of `field` (device inputs as elrt_solve_field) with
  * every candidate (local_chunk in {0, 512, 1024, ...} below the field's element count, lu_pairs in

@@ -12,8 +12,9 @@
 //   k_rowcol           (blocks of 128 rows or columns per element): L21 from L21 U11 = A21 written
 //                      back to the matrix; U12 from L11 U12 = A12 written back to the matrix and,
 //                      transposed (K-major), to one side buffer whose rows hold both panels of the
-//                      pair (FP32 values and their low TF32 parts, or FP16 high parts and FP16
-//                      remainders).  On the right-hand-side columns this is the forward substitution;
+//                      pair as FP32 values and their low TF32 parts, or four panels as FP16 high parts
+//                      and FP16 remainders.  On the right-hand-side columns this is the forward
+//                      substitution;
 //   k_tc_update<NK, H> (tensor cores): C -= L21 U12 with three products hi*hi + hi*lo + lo*hi of
 //                      TF32 parts or (H, when the entries fit FP16's range: the factorisation and
 //                      the re-solves' forward sweeps, their residuals scaled per element) FP16
@@ -21,11 +22,16 @@
 //                      per instruction against 8).  Panel a is applied with rank 64 to panel b's
 //                      columns and rows only; once panel b is factored, the rest of the matrix
 //                      takes both panels in one rank-128 update, which moves the C tiles half as
-//                      often as two rank-64 updates.  The FP32 operands come in by TMA (U12^T from
+//                      often as two rank-64 updates; with FP16 parts the first of two pairs is
+//                      applied to the second's columns and rows only, and the rest takes all four
+//                      panels in one rank-256 update.  What bounds all of them is the C traffic (8
+//                      bytes per entry against 2 NK useful flops), so the number of passes over C is
+//                      what counts: 4096 elements at p = 6, N = 16, factorisation and backward sweep,
+//                      rank 128 15.0 ms, rank 128 and 256 13.0 ms.  The FP32 operands come in by TMA (U12^T from
 //                      the side buffer, C from the matrix); the L21 strip goes straight from the
 //                      matrix into tensor memory as TF32 (or FP16) high and low parts.
-// Panels left over after the pairs (nu not a multiple of 128) are factored one at a time with
-// rank-64 updates; in the backward sweeps a last partial panel joins the panel before it.  The
+// Panels left over are factored in pairs, then one at a time with rank-64 updates; in the backward
+// sweeps a last partial panel joins the panels before it.  The
 // backward substitution and the forward/backward sweeps of the refinement re-solves reuse the
 // stored factors (L21 and U12 in the matrix, the diagonal blocks) with the same kernels.
 #include <math.h>
@@ -46,10 +52,11 @@ constexpr int NBP = 64;     // panel width
 constexpr int UTK = 256;    // row of the U12^T side buffer: two consecutive panels (K 0 .. 127), then
                             // the low TF32 parts of the same values (K 128 .. 255)
 constexpr int UTL = 128;    // K offset of the low parts
-// FP16 side buffer (updates with 3xFP16 products): a row holds the FP16 high parts of both panels
-// (K 0 .. 127), then the FP16 rounding of the remainders (K 128 .. 255), 512 bytes
-constexpr int UTK16 = 256;
-constexpr int UTL16 = 128;
+// FP16 side buffer (updates with 3xFP16 products): a row holds the FP16 high parts of four panels
+// (K 0 .. 255), then the FP16 rounding of the remainders (K 256 .. 511), the same 1024 bytes
+constexpr int UTK16 = 512;
+constexpr int UTL16 = 256;
+static_assert(UTK16 * 2 == UTK * 4, "both formats share the allocation");
 constexpr int UBN = 64;     // trailing-update tile width (N of the MMAs)
 constexpr int UCB = UBN / 32;  // 32-column (128-byte) boxes of a C tile
 
@@ -445,9 +452,9 @@ __device__ __forceinline__ void mma_tf32_ta(uint32_t d_tmem, uint32_t a_tmem, ui
 }
 
 
-// Persistent trailing update C -= L U of rank NK = 64 (one panel) or 128 (two consecutive panels,
-// the second already factored against the first; H: FP16 operands, as the notes after the role
-// list say): one CTA per SM walks the work items (element,
+// Persistent trailing update C -= L U of rank NK = 64 (one panel), 128 or 256 (two or, with FP16
+// operands, four consecutive panels, each already factored against those before it; H: FP16
+// operands, as the notes after the role list say): one CTA per SM walks the work items (element,
 // 128-row strip) of the launch, the strips of one element consecutively (their U12^T tiles are
 // shared through L2).  The L21 strip of an item (columns J .. J+NK-1 of its 128 rows, FP32,
 // straight from the matrix) lives in tensor memory as TF32 high and low parts, in 64-column halves
@@ -467,9 +474,9 @@ __device__ __forceinline__ void mma_tf32_ta(uint32_t d_tmem, uint32_t a_tmem, ui
 //                M = 128, N = 64, K = 8, A from tensor memory) into one of two TMEM accumulators;
 //   warps 2-5,   epilogue: accumulator (tcgen05.ld) and staged C tile -> C - L U, written back
 //   10-13        into the staged tile (warps 2-5 the first 32-column box, 10-13 the second);
-//   warp 14      stores each finished tile with TMA tensor stores (the store map's extents are
-//                r_end rows and c_end columns, so rows and columns outside the update are
-//                clipped) and releases the C stage once the store has read it;
+//   warp 14      stores each finished tile with TMA tensor stores (the map's extents are r_end
+//                rows and c_end columns, so rows and columns outside the update are neither loaded
+//                nor stored) and releases the C stage once the store has read it;
 //   warps 6-9    strip preparation: each thread loads one row of a strip half (columns at or
 //                beyond jb are 0) into registers, waits for a free slot, splits the row and
 //                writes it to its TMEM lane (tcgen05.st).
@@ -477,7 +484,9 @@ __device__ __forceinline__ void mma_tf32_ta(uint32_t d_tmem, uint32_t a_tmem, ui
 // for the first panel, 64 for the second, their low parts UTL further); an NK = 64 update reads
 // the half at K offset koff.  With H the side buffer is FP16 ([E][ld][UTK16], the FP16 roundings
 // and those of the remainders), the strip preparation packs two FP16 values per TMEM column, and
-// an MMA covers K = 16 with the same TMEM-column and descriptor strides as a TF32 one of K = 8.  Every wait is bounded; on a timeout the CTA records a code in *err,
+// an MMA covers K = 16 with the same TMEM-column and descriptor strides as a TF32 one of K = 8; a strip
+// part takes 64 columns of tensor memory, six of them fit, and NK = 256 uses the shared memory of TF32's
+// 128.  Every wait is bounded; on a timeout the CTA records a code in *err,
 // stops issuing work, lets its copies land and frees its TMEM.
 template <int NK, bool H = false>
 struct UpdCfg {
@@ -490,20 +499,22 @@ struct UpdCfg {
     static constexpr int C_STAGE = UCB * C_BOX;
     static constexpr int NU = NK == 64 ? 4 : 2;    // U stages
     static constexpr int NC = 3;                   // C stages
-    static constexpr int NH = NK / 64;             // 64-column strip halves per item
+    static constexpr int NH = NK / 64;             // 64-column strip parts per item
+    // tensor memory: accumulators at columns [0, 2 UBN); then the strip slots, the high part of a 64-column
+    // strip part and its low part: 64 columns each in TF32, 32 in FP16 (two values a column)
+    static constexpr int SLOTS = H ? 6 : 3;
+    static constexpr uint32_t PART = H ? 32 : 64;
+    static __host__ __device__ constexpr uint32_t slot_col(int s, int lo) {
+        return (uint32_t)(2 * UBN) + 2 * PART * (uint32_t)s + PART * (uint32_t)lo;
+    }
+    static_assert(SLOTS >= NH && 2 * UBN + 2 * PART * SLOTS <= 512, "tensor memory");
     static constexpr int BYTES = NU * U_STAGE + NC * C_STAGE;
     static constexpr int TOTAL = BYTES + 1024 + 512;
 };
 static_assert(UpdCfg<64>::TOTAL <= 227 * 1024 && UpdCfg<128>::TOTAL <= 227 * 1024 &&
-                  UpdCfg<64, true>::TOTAL <= 227 * 1024 && UpdCfg<128, true>::TOTAL <= 227 * 1024,
+                  UpdCfg<64, true>::TOTAL <= 227 * 1024 && UpdCfg<128, true>::TOTAL <= 227 * 1024 &&
+                  UpdCfg<256, true>::TOTAL <= 227 * 1024,
               "trailing-update shared memory");
-// tensor memory: accumulators at columns [0, 2 UBN); strip slot s (of kSlots): the high part of a
-// 64-column half at 2 UBN + 128 s, its low part 64 columns further
-constexpr int kSlots = 3;
-__host__ __device__ constexpr uint32_t slot_col(int s, int lo) {
-    return (uint32_t)(2 * UBN) + 128u * (uint32_t)s + 64u * (uint32_t)lo;
-}
-static_assert(slot_col(kSlots - 1, 1) + 64 <= 512, "tensor memory");
 static_assert(UCB == 2, "two epilogue warp groups, one per 32-column box of a C tile");
 constexpr int kStripThreads = 480;
 constexpr int kEpiWarps = 8;
@@ -515,12 +526,11 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 
 template <int NK, bool H>
 __global__ void __launch_bounds__(kStripThreads, 1)
-    k_tc_update(const __grid_constant__ CUtensorMap tM, const __grid_constant__ CUtensorMap tU,
-                const __grid_constant__ CUtensorMap tS, float* __restrict__ Mall, int nu, int64_t ld, int64_t estride,
+    k_tc_update(const __grid_constant__ CUtensorMap tU, const __grid_constant__ CUtensorMap tS, float* __restrict__ Mall, int nu, int64_t ld, int64_t estride,
                 int64_t E, int J, int jb, int koff, int r0, int r_end, int c0, int c_end, int* __restrict__ err,
                 const double* __restrict__ res_max) {
     using Cfg = UpdCfg<NK, H>;
-    constexpr int NU = Cfg::NU, NC = Cfg::NC, NH = Cfg::NH, KB = Cfg::KB, KW = Cfg::KW;
+    constexpr int NU = Cfg::NU, NC = Cfg::NC, NH = Cfg::NH, KB = Cfg::KB, KW = Cfg::KW, kSlots = Cfg::SLOTS;
     constexpr int ULO = H ? UTL16 : UTL;  // K offset of the low parts in the side buffer
     extern __shared__ __align__(1024) unsigned char ssm_raw[];
     unsigned char* base = (unsigned char*)(((uintptr_t)ssm_raw + 1023) & ~(uintptr_t)1023);
@@ -597,7 +607,7 @@ __global__ void __launch_bounds__(kStripThreads, 1)
                 }
                 unsigned char* cs = cstage0 + sc * Cfg::C_STAGE;
                 tc::mbar_expect_tx(&c_full[sc], Cfg::C_STAGE);
-                for (int cb = 0; cb < UCB; ++cb) tma_load_3d(&tM, &c_full[sc], cs + cb * Cfg::C_BOX, n0 + 32 * cb, m0, (int)e);
+                for (int cb = 0; cb < UCB; ++cb) tma_load_3d(&tS, &c_full[sc], cs + cb * Cfg::C_BOX, n0 + 32 * cb, m0, (int)e);
                 ++issued_c;
             }
         }
@@ -633,7 +643,7 @@ __global__ void __launch_bounds__(kStripThreads, 1)
                         }
                         tc::tc_fence_after();
                     }
-                    const uint32_t a_hi = tmem + slot_col(sl, 0), a_lo = tmem + slot_col(sl, 1);
+                    const uint32_t a_hi = tmem + Cfg::slot_col(sl, 0), a_lo = tmem + Cfg::slot_col(sl, 1);
                     if constexpr (H) {  // one 64-wide K box per half; K = 16 per instruction (8 TMEM columns, 32 bytes)
                         const uint64_t bh = tc::sw128_desc(tc::smem_u32(us + j * Cfg::U_BOX));
                         const uint64_t bl = tc::sw128_desc(tc::smem_u32(us + (KB + j) * Cfg::U_BOX));
@@ -713,8 +723,8 @@ __global__ void __launch_bounds__(kStripThreads, 1)
                         hi[k] = __uint_as_float(pack_h2(h0, h1));
                         lo[k] = __uint_as_float(pack_h2(l0, l1));
                     }
-                    tmem_st32(tmem + lane_off + slot_col(sl, 0), hi);
-                    tmem_st32(tmem + lane_off + slot_col(sl, 1), lo);
+                    tmem_st32(tmem + lane_off + Cfg::slot_col(sl, 0), hi);
+                    tmem_st32(tmem + lane_off + Cfg::slot_col(sl, 1), lo);
                 } else {
 #pragma unroll
                     for (int hh = 0; hh < 2; ++hh) {
@@ -724,8 +734,8 @@ __global__ void __launch_bounds__(kStripThreads, 1)
                             hi[k] = tf32_hi(v[hh * 32 + k]);
                             lo[k] = v[hh * 32 + k] - hi[k];
                         }
-                        tmem_st32(tmem + lane_off + slot_col(sl, 0) + hh * 32, hi);
-                        tmem_st32(tmem + lane_off + slot_col(sl, 1) + hh * 32, lo);
+                        tmem_st32(tmem + lane_off + Cfg::slot_col(sl, 0) + hh * 32, hi);
+                        tmem_st32(tmem + lane_off + Cfg::slot_col(sl, 1) + hh * 32, lo);
                     }
                 }
                 tmem_st_wait();
@@ -837,7 +847,7 @@ __global__ void __launch_bounds__(kStripThreads, 1)
             }
             // and let the strip-slot commits issued after it arrive before the CTA's shared memory goes
             const int items = (int)((W - 1 - blockIdx.x) / gridDim.x) + 1;
-            for (int h = (items - 1) * NH; committed == items * ntile && h < items * NH; ++h) {
+            for (int h = max(0, items * NH - kSlots); committed == items * ntile && h < items * NH; ++h) {
                 const long long t1 = clock64();
                 while (!tc::mbar_try_wait(&s_empty[h % kSlots], (h / kSlots) & 1) && clock64() - t1 < tc::kWaitCycles / 4) {
                 }
@@ -905,7 +915,7 @@ bool mapM(CUtensorMap* m, const float* M, int64_t rows, int64_t cols, int64_t ld
 }
 
 struct TcMaps {
-    CUtensorMap m, u;
+    CUtensorMap u;
     bool f16;  // trailing updates with 3xFP16 products (FP16 side buffer), else 3xTF32
     const double* res_max = nullptr;  // per-element residual maxima of a scaled FP16 re-solve
 };
@@ -921,16 +931,16 @@ elrt_status update(elrt_ctx* ctx, const TcMaps& mp, float* M, int64_t ld, int64_
     if (r_end <= r0 || c_end <= c0) return ELRT_OK;
     const double R = r_end - r0, C = c_end - c0;
     ProfScope ps(ctx, "lu_tc_update", 1, (double)E * (8.0 * R * C + 4.0 * (R + C) * jb), (double)E * 2.0 * R * C * jb);
-    CUtensorMap tS;  // stores: rows [0, r_end), columns [0, c_end)
+    CUtensorMap tS;  // rows [0, r_end), columns [0, c_end): what lies outside is neither loaded nor stored
     if (!mapM(&tS, M, r_end, c_end, ld, estride, E)) return ctx_fail(ctx, ELRT_EINVAL, "tensor map encoding failed");
     const int64_t items = (int64_t)((r_end - r0 + 127) / 128) * E;
     const unsigned grid = (unsigned)std::min<int64_t>(items, ctx->sms);
     if (mp.f16)
         k_tc_update<NK, true><<<grid, kStripThreads, UpdCfg<NK, true>::TOTAL, ctx->stream>>>(
-            mp.m, mp.u, tS, M, ctx->tab.nu, ld, estride, E, J, jb, koff, r0, r_end, c0, c_end, err, mp.res_max);
-    else
+            mp.u, tS, M, ctx->tab.nu, ld, estride, E, J, jb, koff, r0, r_end, c0, c_end, err, mp.res_max);
+    else if constexpr (NK <= 128)
         k_tc_update<NK, false><<<grid, kStripThreads, UpdCfg<NK, false>::TOTAL, ctx->stream>>>(
-            mp.m, mp.u, tS, M, ctx->tab.nu, ld, estride, E, J, jb, koff, r0, r_end, c0, c_end, err, nullptr);
+            mp.u, tS, M, ctx->tab.nu, ld, estride, E, J, jb, koff, r0, r_end, c0, c_end, err, nullptr);
     return cuda_check(ctx, cudaGetLastError(), "tc update launch");
 }
 
@@ -952,7 +962,7 @@ elrt_status prepare(elrt_ctx* ctx, float* M, int64_t ld, int64_t estride, const 
     // every column block starts at a multiple of 64 or at nu, and the vector accesses and TMA copies
     // need each to start on a 16-byte boundary (n_angles % 4 == 0 already makes nu a multiple of 4)
     if (nu % 4 != 0 || ld % 4 != 0) return ctx_fail(ctx, ELRT_EINVAL, "tensor-core LU needs nu and ld multiples of 4");
-    if (!mapM(&mp->m, M, nu, ld, ld, estride, E) || !(f16 ? map3_16(&mp->u, Ut, ld, E, UBN) : map3(&mp->u, Ut, ld, E, UBN)))
+    if (!(f16 ? map3_16(&mp->u, Ut, ld, E, UBN) : map3(&mp->u, Ut, ld, E, UBN)))
         return ctx_fail(ctx, ELRT_EINVAL, "tensor map encoding failed");
     static bool attr_done = false;
     if (!attr_done) {
@@ -967,6 +977,9 @@ elrt_status prepare(elrt_ctx* ctx, float* M, int64_t ld, int64_t estride, const 
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_tc_update<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      UpdCfg<128, true>::TOTAL);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_tc_update<256, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     UpdCfg<256, true>::TOTAL);
         if (e != cudaSuccess) return cuda_check(ctx, e, "smem attribute");
         attr_done = true;
     }
@@ -1014,6 +1027,41 @@ elrt_status rowcol(elrt_ctx* ctx, const TcMaps& mp, float* M, int64_t ld, int64_
     return cuda_check(ctx, cudaGetLastError(), "rowcol launch");
 }
 
+// The same with 3xFP16 products: groups of four panels from the bottom, the first with the last partial panel.
+// Within a group (panels c0 > c1 > c2 > c3) X_c0, the rank-64 update of c1's rows, X_c1, the rank-128 update of
+// the rows of c2 and c3, X_c2, the rank-64 update of c3's rows, X_c3; then one rank-256 update of the rows
+// above the group.  Panel c_i lies at side-buffer offset 64 (3 - i), zero beyond a partial panel's width; only
+// the topmost group may have fewer panels, and has no rows above it.
+elrt_status backward_fours(elrt_ctx* ctx, const TcMaps& mp, float* M, int64_t ld, int64_t estride, int64_t E,
+                           const float* Tinv, float* Ut, int* err, int nin) {
+    const int nu = ctx->tab.nu, c_end = nu + nin;
+    for (int top = nu; top > 0;) {
+        int c[4], n = 0;
+        for (int e = top; n < 4 && e > 0; e = c[n++]) c[n] = (e - 1) / NBP * NBP;
+        auto solve = [&](int i) {
+            return rowcol(ctx, mp, M, ld, estride, E, c[i], (i ? c[i - 1] : top) - c[i], Tinv, 0, 0, nu, c_end, 1, Ut,
+                          NBP * (n - 1 - i));
+        };
+        elrt_status s = solve(0);
+        if (!s && n > 1) {
+            s = update<64>(ctx, mp, M, ld, estride, E, c[0], top - c[0], NBP * (n - 1), c[1], c[0], nu, c_end, err);
+            if (!s) s = solve(1);
+        }
+        if (!s && n > 2) {
+            s = update<128>(ctx, mp, M, ld, estride, E, c[1], top - c[1], NBP * (n - 2), c[n - 1], c[1], nu, c_end, err);
+            if (!s) s = solve(2);
+        }
+        if (!s && n > 3) {
+            s = update<64>(ctx, mp, M, ld, estride, E, c[2], NBP, NBP * (n - 3), c[3], c[2], nu, c_end, err);
+            if (!s) s = solve(3);
+            if (!s) s = update<256>(ctx, mp, M, ld, estride, E, c[3], top - c[3], 0, 0, c[3], nu, c_end, err);
+        }
+        if (s) return s;
+        top = c[n - 1];
+    }
+    return ELRT_OK;
+}
+
 // backward substitution on the right-hand-side columns: X_J = U11^{-1} X_J, then the rows above
 // lose U[0..J, J..J+jb) X_J.  With the pair schedule, per pair (a, b), last pair first: X_b, the
 // rank-64 update of panel a's rows, X_a, and one rank-128 update of the rows above the pair (both
@@ -1023,6 +1071,7 @@ elrt_status rowcol(elrt_ctx* ctx, const TcMaps& mp, float* M, int64_t ld, int64_
 elrt_status backward_sweep_tc(elrt_ctx* ctx, const TcMaps& mp, float* M, int64_t ld, int64_t estride, int64_t E,
                               const float* Tinv, float* Ut, int* err, int nin) {
     const int nu = ctx->tab.nu;
+    if (mp.f16 && ctx->tune.lu_pairs) return backward_fours(ctx, mp, M, ld, estride, E, Tinv, Ut, err, nin);
     const int npair = ctx->tune.lu_pairs ? nu / (2 * NBP) : 0;
     const int rem = nu - 2 * NBP * npair;  // columns beyond the last pair
     if (npair > 0 && rem > 0 && rem <= NBP) {
@@ -1097,18 +1146,35 @@ elrt_status tc_lu_factor_solve(elrt_ctx* ctx, float* M, int64_t ld, int64_t estr
     elrt_status s = prepare(ctx, M, ld, estride, sd.Ut, E, &mp, f16);
     if (s) return s;
     int J = 0;
-    // pairs of full panels a = [J, J+64), b = [J+64, J+128): panel a is factored and applied to
-    // panel b's columns and rows only (two narrow rank-64 updates), panel b is factored, and the
-    // rest of the matrix takes both in one rank-128 update (half the C traffic of two rank-64 ones)
-    for (; ctx->tune.lu_pairs && J + 2 * NBP <= nu; J += 2 * NBP) {
+    // a pair of full panels a = [J, J+64), b = [J+64, J+128), in the side buffer at K offsets koff and koff +
+    // 64: panel a is factored and applied to panel b's columns and rows only (two narrow rank-64 updates),
+    // panel b is factored; the rest of the matrix is the caller's
+    auto factor_pair = [&](int J, int koff) {
         const int Jb = J + NBP, Jn = J + 2 * NBP;
         diag_block(ctx, M, ld, estride, E, J, NBP, sd.Tinv, estat);
-        s = rowcol(ctx, mp, M, ld, estride, E, J, NBP, sd.Tinv, Jb, nu, Jb, ncols, 0, sd.Ut, 0);
-        if (!s) s = update<64>(ctx, mp, M, ld, estride, E, J, NBP, 0, Jb, nu, Jb, Jn, err);
-        if (!s) s = update<64>(ctx, mp, M, ld, estride, E, J, NBP, 0, Jb, Jn, Jn, ncols, err);
+        elrt_status s = rowcol(ctx, mp, M, ld, estride, E, J, NBP, sd.Tinv, Jb, nu, Jb, ncols, 0, sd.Ut, koff);
+        if (!s) s = update<64>(ctx, mp, M, ld, estride, E, J, NBP, koff, Jb, nu, Jb, Jn, err);
+        if (!s) s = update<64>(ctx, mp, M, ld, estride, E, J, NBP, koff, Jb, Jn, Jn, ncols, err);
         if (s) return s;
         diag_block(ctx, M, ld, estride, E, Jb, NBP, sd.Tinv, estat);
-        s = rowcol(ctx, mp, M, ld, estride, E, Jb, NBP, sd.Tinv, Jn, nu, Jn, ncols, 0, sd.Ut, NBP);
+        return rowcol(ctx, mp, M, ld, estride, E, Jb, NBP, sd.Tinv, Jn, nu, Jn, ncols, 0, sd.Ut, koff + NBP);
+    };
+    // with 3xFP16 products, two pairs at a time: the first is applied with rank 128 to the second's columns
+    // and rows only, and the rest takes all four panels in one rank-256 update (half the C traffic of two
+    // rank-128 ones; 3xTF32 operands leave no room for four panels in tensor memory)
+    for (; f16 && ctx->tune.lu_pairs && J + 4 * NBP <= nu; J += 4 * NBP) {
+        const int Jm = J + 2 * NBP, Jn = J + 4 * NBP;
+        s = factor_pair(J, 0);
+        if (!s) s = update<128>(ctx, mp, M, ld, estride, E, J, 2 * NBP, 0, Jm, nu, Jm, Jn, err);
+        if (!s) s = update<128>(ctx, mp, M, ld, estride, E, J, 2 * NBP, 0, Jm, Jn, Jn, ncols, err);
+        if (!s) s = factor_pair(Jm, 2 * NBP);
+        if (!s) s = update<256>(ctx, mp, M, ld, estride, E, J, 4 * NBP, 0, Jn, nu, Jn, ncols, err);
+        if (s) return s;
+    }
+    // pairs: the rest of the matrix takes both panels in one rank-128 update
+    for (; ctx->tune.lu_pairs && J + 2 * NBP <= nu; J += 2 * NBP) {
+        const int Jn = J + 2 * NBP;
+        s = factor_pair(J, 0);
         if (!s) s = update<128>(ctx, mp, M, ld, estride, E, J, 2 * NBP, 0, Jn, nu, Jn, ncols, err);
         if (s) return s;
     }
@@ -1138,13 +1204,27 @@ elrt_status tc_lu_resolve(elrt_ctx* ctx, float* M, int64_t ld, int64_t estride, 
     if (s) return s;
     if (f16_fwd) mp.res_max = res_max;
     int J = 0;
-    // forward substitution with the unit lower factor, in the factorisation's panel pairs: X_a, the
-    // rank-64 update of panel b's rows, X_b, one rank-128 update of the rows below the pair
-    for (; ctx->tune.lu_pairs && J + 2 * NBP <= nu; J += 2 * NBP) {
+    // forward substitution with the unit lower factor, in the factorisation's panel groups: X_a, the rank-64
+    // update of panel b's rows, X_b, and one rank-128 update of the rows below the pair, or (3xFP16) of the
+    // next pair's rows, that pair, and one rank-256 update of the rows below both
+    auto solve_pair = [&](int J, int koff) {
         const int Jb = J + NBP, Jn = J + 2 * NBP;
-        s = rowcol(ctx, mp, M, ld, estride, E, J, NBP, sd.Tinv, 0, 0, nu, nu + nin, 0, sd.Ut, 0);
-        if (!s) s = update<64>(ctx, mp, M, ld, estride, E, J, NBP, 0, Jb, Jn, nu, nu + nin, err);
-        if (!s) s = rowcol(ctx, mp, M, ld, estride, E, Jb, NBP, sd.Tinv, 0, 0, nu, nu + nin, 0, sd.Ut, NBP);
+        elrt_status s = rowcol(ctx, mp, M, ld, estride, E, J, NBP, sd.Tinv, 0, 0, nu, nu + nin, 0, sd.Ut, koff);
+        if (!s) s = update<64>(ctx, mp, M, ld, estride, E, J, NBP, koff, Jb, Jn, nu, nu + nin, err);
+        if (!s) s = rowcol(ctx, mp, M, ld, estride, E, Jb, NBP, sd.Tinv, 0, 0, nu, nu + nin, 0, sd.Ut, koff + NBP);
+        return s;
+    };
+    for (; f16_fwd && ctx->tune.lu_pairs && J + 4 * NBP <= nu; J += 4 * NBP) {
+        const int Jm = J + 2 * NBP, Jn = J + 4 * NBP;
+        s = solve_pair(J, 0);
+        if (!s) s = update<128>(ctx, mp, M, ld, estride, E, J, 2 * NBP, 0, Jm, Jn, nu, nu + nin, err);
+        if (!s) s = solve_pair(Jm, 2 * NBP);
+        if (!s) s = update<256>(ctx, mp, M, ld, estride, E, J, 4 * NBP, 0, Jn, nu, nu, nu + nin, err);
+        if (s) return s;
+    }
+    for (; ctx->tune.lu_pairs && J + 2 * NBP <= nu; J += 2 * NBP) {
+        const int Jn = J + 2 * NBP;
+        s = solve_pair(J, 0);
         if (!s) s = update<128>(ctx, mp, M, ld, estride, E, J, 2 * NBP, 0, Jn, nu, nu, nu + nin, err);
         if (s) return s;
     }
