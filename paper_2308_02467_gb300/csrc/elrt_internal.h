@@ -164,6 +164,7 @@ elrt_status global_recover_rows(elrt_ctx* ctx, int nx, int nz, int rows, const v
 
 // ---- sweep preconditioner of the skeleton GMRES (sweep.cu)
 void sweep_orders(int nx, int nz, int* out);                 // [4 E] work items in their global order
+bool sweep_needs_order(const Tab& t, int nx, int nz, int sms);  // whether an application reads them
 size_t sweep_words_bytes(const Tab& t, int64_t E);          // scratch of one application's outflow words
 elrt_status sweep_apply(elrt_ctx* ctx, int nx, int nz, const void* A, int a_bytes, const float* u, float* z,
                         const int* order, void* zw, int* flags, const int* done, const int* nsteps);

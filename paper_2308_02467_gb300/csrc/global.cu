@@ -1518,7 +1518,7 @@ elrt_status gmres(elrt_ctx* ctx, int nx, int nz, const void* Aop, const double* 
     GmState* hst = (GmState*)ctx->h_pinned;
     const int rows = t.nin;
 
-    if (pc) {
+    if (pc && sweep_needs_order(t, nx, nz, ctx->sms)) {
         std::vector<int> ord((size_t)4 * E);
         sweep_orders(nx, nz, ord.data());
         s = cuda_check(ctx, cudaMemcpyAsync(pc_order, ord.data(), ord.size() * sizeof(int), cudaMemcpyHostToDevice, sm),

@@ -298,6 +298,290 @@ __global__ void __launch_bounds__(kSwThreads, 1) k_sweep(SweepArgs a, const AT* 
     }
 }
 
+// ------------------------------------------------------------------------------------------------
+// The same application with a mesh line per pair of CTAs, for meshes whose shorter side has at most half as
+// many lines as there are SMs.
+//
+// What bounds k_sweep is its dependency chain: every element step waits for values that another CTA has just
+// written, ~1 us through L2 beside ~1 us of work.  Here the lines along the longer side of the mesh (rows iz
+// when nx >= nz, else columns) are dealt out, two CTAs each: CTA 0 of a line computes the outflow of the
+// "along" faces, which only the next element of the same line waits for -- it passes from step to step through
+// shared memory -- and CTA 1 the "cross" faces, towards the next line.  Both walk the line's elements in each
+// sweep's order, sweep after sweep.  Everything else an item reads (the cross inflow, the values of earlier
+// sweeps, and for CTA 1 the along inflow) was written a step or more earlier and is polled ahead of time: four
+// gather warps fetch the inflow of the next four items into their own buffers while the compute warps, eight rows
+// each, run the current one, and one thread keeps the operator ring full: the L2 latency is paid once per line,
+// not once per element.  A step's operator rows are in registers before it starts, so its chain is the inflow
+// load, the products, nine shuffles and a barrier; with four rows per warp the step was bound by its warps'
+// instructions instead.  Measured per application against k_sweep (us): 64 x 64 elements at p = 6, N = 16,
+// 584 -> 446; 76 x 76, 689 -> 551; 32 x 32, 290 -> 213; 24 x 41, 278 -> 254; 127 x 17 at p = 4, 651 -> 370; 37 x 52,
+// 358 -> 295; 16 x 23 at p = 8, 279 -> 196.  At 64 x 64 it reads 3.7 TB/s.  The words, their slots and the
+// arithmetic of a value are k_sweep's (per-lane column pairs, butterfly over the lanes in the order 16, 8, 4, 2,
+// 1), so the result is the same bits.  Each CTA's order is consistent with (sweep, wavefront), every item waits
+// only for items before it in that order, and all CTAs are resident: no deadlock.  Every wait is bounded.
+// The operator rows of one face and item come through a ring of bulk copies as before.
+constexpr int kLnBufs = 4;    // inflow buffers, one gather warp each
+constexpr int kLnStages = 4;  // operator stages at most
+constexpr int kLnMaxIn = 320;
+__host__ __device__ constexpr int ln_warps(int nf) { return (nf + 7) / 8; }  // compute warps
+constexpr int kLnThreads = 32 * (ln_warps(kLnMaxIn / 4) + kLnBufs + 1);      // at most, with the copy warp
+
+// mbar_wait with the common case, a phase already complete, first
+__device__ __forceinline__ bool ready(uint64_t* bar, uint32_t parity, volatile int* abort) {
+    return tc::mbar_try_wait(bar, parity) || tc::mbar_wait(bar, parity, abort);
+}
+__device__ __forceinline__ void arrive(uint64_t* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar)) : "memory");
+}
+
+template <typename AT, int NP>
+__global__ void __launch_bounds__(kLnThreads, 1) k_sweep_lines(SweepArgs a, const AT* __restrict__ A) {
+    if ((a.done && *a.done) || (a.nsteps && *a.nsteps == 0)) return;
+    extern __shared__ __align__(128) unsigned char sw_smem[];
+    const int nin = a.nin, nf = a.nface, npair = nin / 2, NS = a.stages;
+    const int blk = nf * nin;  // operator entries of an item: one face's rows
+    AT* stage0 = reinterpret_cast<AT*>(sw_smem);
+    float* xin0 = reinterpret_cast<float*>(sw_smem + (size_t)NS * blk * sizeof(AT));
+    __shared__ uint64_t full[kLnStages], gat[kLnBufs], rel[kLnBufs];
+    __shared__ int abort_s;
+    volatile int* abort = &abort_s;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int ax = a.nx >= a.nz ? 0 : 1;  // lines along x or z
+    const int L = ax == 0 ? a.nx : a.nz, line = blockIdx.x >> 1, role = blockIdx.x & 1;
+    const int kf = role == 0 ? ax : 1 - ax;  // which downwind face of a sweep this CTA computes (sw_down)
+    const int cw = ln_warps(nf), xb = nin + nf;  // an inflow buffer: the inflow, then the rows' right-hand sides
+    const int total = 4 * L;                 // items n = sweep * L + i, i the element's place in the sweep's order
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < NS; ++i) tc::mbar_init(&full[i], 1);
+        for (int i = 0; i < kLnBufs; ++i) {
+            tc::mbar_init(&gat[i], 1);
+            tc::mbar_init(&rel[i], 1);
+        }
+        tc::fence_barrier_init();
+        abort_s = 0;
+    }
+    __syncthreads();
+    // a sweep's first element on this line and the step to its next one; sweeps 0 and 3 run along +x, 0 and 1
+    // along +z
+    const int stride = ax == 0 ? 1 : a.nx, e_low = ax == 0 ? a.nx * line : line;
+    auto forward = [&](int c) { return ax == 0 ? (c == 0 || c == 3) : c <= 1; };
+    auto first = [&](int c) { return forward(c) ? e_low : e_low + (L - 1) * stride; };
+    auto step = [&](int c) { return forward(c) ? stride : -stride; };
+    auto give_up = [&]() {
+        atomicOr(a.err, 1);
+        *(volatile int*)a.abort = 1;
+        *abort = 1;
+    };
+    if (warp < cw) {
+        // a wait that gives up sets abort, after which no wait waits: every warp runs all its (then meaningless)
+        // steps, so the block barrier always has its count
+        const int r0 = 8 * warp, nr = min(8, nf - r0);
+        const int rl = lane >> 2;  // row r0 + rl is this lane's (one lane of four writes it)
+        int col[NP];               // entries 2 (lane + 32 q) of a row, clamped; beyond the row x is zero
+        bool in[NP];
+#pragma unroll
+        for (int q = 0; q < NP; ++q) {
+            in[q] = lane + 32 * q < npair;
+            col[q] = 2 * min(lane + 32 * q, npair - 1);
+        }
+        const bool writes = (lane & 3) == 0 && rl < nr;
+        // this warp's rows in operator stage st (rows beyond the face's repeat its last one)
+        float2 av[8][NP];
+        auto load_a = [&](int st) {
+            const AT* Ar = stage0 + st * blk + r0 * nin;
+#pragma unroll
+            for (int kk = 0; kk < 8; ++kk) {
+#pragma unroll
+                for (int q = 0; q < NP; ++q) av[kk][q] = ld_pair(Ar, col[q]);
+                if (kk + 1 < nr) Ar += nin;
+            }
+        };
+        if (!ready(&full[0], 0, abort) && !*abort) give_up();
+        load_a(0);
+        int st = 0, n = 0, b = 0;
+        uint32_t sph = 0, bph = 0;  // operator stage and inflow buffer, and the parities of their phases
+        for (int c = 0; c < 4; ++c) {
+            const int F = sw_down(c, kf), de = step(c);
+            const bool last = sw_last(F) == c;
+            const int nxt_off = ((F + 2) & 3) * nf + r0 + rl;
+            VerVal* zp = a.zw + ((int64_t)c * a.E + first(c)) * npair + kf * nf + r0 + rl;
+            float* zo = a.z + (int64_t)first(c) * nin + F * nf + r0 + rl;
+            for (int i = 0; i < L; ++i, ++n) {
+                if (!ready(&gat[b], bph, abort) && !*abort) give_up();
+                const float* xin = xin0 + b * xb;
+                const float uv = xin[nin + r0 + min(rl, nr - 1)];
+                float2 xv[NP];
+#pragma unroll
+                for (int q = 0; q < NP; ++q) {
+                    xv[q] = *reinterpret_cast<const float2*>(xin + col[q]);
+                    if (!in[q]) xv[q] = make_float2(0.f, 0.f);
+                }
+                float v[8];
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk) v[kk] = 0.f;
+#pragma unroll
+                for (int q = 0; q < NP; ++q)
+#pragma unroll
+                    for (int kk = 0; kk < 8; ++kk) {
+                        v[kk] = fmaf(av[kk][q].x, xv[q].x, v[kk]);
+                        v[kk] = fmaf(av[kk][q].y, xv[q].y, v[kk]);
+                    }
+                const float val = uv + warp_sum8(v, lane);
+                const int b1 = (b + 1) % kLnBufs;
+                if (writes) {
+                    // the next element of the line takes the along values through its inflow buffer
+                    if (role == 0 && i + 1 < L) xin0[b1 * xb + nxt_off] = val;
+                    st_verval(zp, val, 1);
+                    if (last) *zo = val;
+                }
+                // the step is over in every compute warp: stage and buffer are free (the stage's rows are in
+                // registers), the next inflow is complete
+                asm volatile("bar.sync 1, %0;" ::"r"(32 * cw) : "memory");
+                if (threadIdx.x == 0) arrive(&rel[b]);
+                if (++st == NS) {
+                    st = 0;
+                    sph ^= 1;
+                }
+                b = b1;
+                if (b == 0) bph ^= 1;
+                zp += (int64_t)de * npair;
+                zo += (int64_t)de * nin;
+                if (n + 1 < total) {  // the next item's operator rows (before the reduction: slower)
+                    if (!ready(&full[st], sph, abort) && !*abort) give_up();
+                    load_a(st);
+                }
+            }
+        }
+    } else if (warp == cw + kLnBufs) {
+        // operator copies: item n + NS once step n is over
+        if (lane == 0) {
+            const int bytes = blk * (int)sizeof(AT);
+            int c = 0, i = 0, issued = 0, st = 0;
+            auto issue = [&]() {
+                const unsigned char* src = reinterpret_cast<const unsigned char*>(
+                    A + ((int64_t)(first(c) + i * step(c)) * nin + sw_down(c, kf) * nf) * nin);
+                unsigned char* dst = reinterpret_cast<unsigned char*>(stage0 + (size_t)st * blk);
+                tc::mbar_expect_tx(&full[st], (uint32_t)bytes);
+                for (int off = 0; off < bytes; off += kSwChunk)
+                    tc::bulk_load(dst + off, src + off, (uint32_t)min(kSwChunk, bytes - off), &full[st]);
+                if (++st == NS) st = 0;
+                if (++i == L) {
+                    i = 0;
+                    ++c;
+                }
+                ++issued;
+            };
+            while (issued < NS && issued < total) issue();
+            for (int n = 0; n + NS < total; ++n) {
+                if (!ready(&rel[n % kLnBufs], (n / kLnBufs) & 1, abort) || *abort) break;
+                issue();
+            }
+            // let the copies this CTA issued land before it exits (bounded)
+            for (int q = max(0, issued - NS); q < issued; ++q) {
+                const long long t0 = clock64();
+                while (!tc::mbar_try_wait(&full[q % NS], (q / NS) & 1) && clock64() - t0 < kSwSpin) {
+                }
+            }
+        }
+    } else {
+        // gather warp g: the inflow of items g, g + 4, ... into buffer g.  Lane entries j = lane + 32 q: inflow
+        // face G = j / nf.  A neighbour through a face that is not one of the sweep's downwind faces is upwind
+        // (this sweep's slot); else the latest earlier sweep's that recomputed its face towards us (none: zero).
+        const int g = warp - cw;
+        const VerVal* w[2 * NP];  // the word of the sweep's first element, nullptr: always zero
+        unsigned up_m = 0, dn_m = 0, own_m = 0;  // bit q: along inflow (none at i = 0), the far along neighbour's (none
+                                                 // at i = L - 1), the face the compute warps fill (CTA 0, i > 0)
+        const float* ub = nullptr;  // right-hand side of the rows of the sweep's first element
+        int de = 0, du = 0;
+        auto sweep = [&](int c) {
+            de = step(c) * npair;
+            du = step(c) * nin;
+            ub = a.u + (int64_t)first(c) * nin + sw_down(c, kf) * nf;
+            up_m = dn_m = own_m = 0;
+#pragma unroll
+            for (int q = 0; q < 2 * NP; ++q) {
+                const int j = lane + 32 * q, G = j / nf, off = j - G * nf, H = (G + 2) & 3;
+                w[q] = nullptr;
+                if (j >= nin) continue;
+                const bool along = (G & 1) != ax;  // faces 1, 3 along x, 0, 2 along z
+                const bool upwind = G != sw_down(c, 0) && G != sw_down(c, 1);
+                const int slot = upwind ? c : sw_prev(c, H);
+                const int dl = G == 1 ? 1 : G == 3 ? -1 : G == 2 ? a.nx : -a.nx;  // the neighbour's element
+                const int ln = line + (G == 1 || G == 2 ? 1 : -1);                 // its line (cross faces)
+                if (slot < 0 || (!along && (ln < 0 || ln >= min(a.nx, a.nz)))) continue;
+                w[q] = a.zw + ((int64_t)slot * a.E + first(c) + dl) * npair + (sw_down(slot, 0) == H ? off : nf + off);
+                if (along) (upwind ? up_m : dn_m) |= 1u << q;
+                if (along && upwind && role == 0) own_m |= 1u << q;
+            }
+        };
+        bool ok = true;
+        int c = -1, cn = 0, i = g;
+        for (int n = g, k = 0; n < total && ok; n += kLnBufs, i += kLnBufs, ++k) {
+            while (i >= L) {
+                i -= L;
+                ++cn;
+            }
+            if (cn != c) sweep(c = cn);
+            if (k > 0) ok = ready(&rel[g], (k - 1) & 1, abort);
+            const unsigned none = (i == 0 ? up_m : 0u) | (i == L - 1 ? dn_m : 0u), own = i > 0 ? own_m : 0u;
+            const int64_t at = (int64_t)i * de;
+            VerVal x[2 * NP];
+#pragma unroll
+            for (int q = 0; q < 2 * NP; ++q) {
+                x[q] = VerVal{0.f, 1};
+                if (w[q] && !(((none | own) >> q) & 1)) x[q] = ld_verval(w[q] + at);
+            }
+            float u[3];  // n_face <= 80
+#pragma unroll
+            for (int q = 0; q < 3; ++q) u[q] = lane + 32 * q < nf ? __ldg(ub + (int64_t)i * du + lane + 32 * q) : 0.f;
+            const long long t0 = clock64();
+            while (ok) {
+                bool miss = false;
+#pragma unroll
+                for (int q = 0; q < 2 * NP; ++q)
+                    if (x[q].ver == 0) {
+                        x[q] = ld_verval(w[q] + at);
+                        miss |= x[q].ver == 0;
+                    }
+                if (!miss) break;
+                if (*abort || *(volatile int*)a.abort || clock64() - t0 > kSwSpin) ok = false;
+            }
+            ok = __all_sync(0xffffffffu, ok);
+#pragma unroll
+            for (int q = 0; q < 2 * NP; ++q) {
+                const int j = lane + 32 * q;
+                if (j < nin && !((own >> q) & 1)) xin0[g * xb + j] = x[q].v;
+            }
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+                if (lane + 32 * q < nf) xin0[g * xb + nin + lane + 32 * q] = u[q];
+            __syncwarp();
+            if (lane == 0 && ok) arrive(&gat[g]);
+        }
+        if (!ok && lane == 0) give_up();
+    }
+}
+
+// Stages of k_sweep_lines for an operator of es-byte entries; 0: it does not take this element or mesh (more
+// lines than CTA pairs fit, where an application is nearer the HBM rate anyway, or rows too wide for two stages
+// or for the registers)
+int line_stages(const Tab& t, int nx, int nz, int es, int sms) {
+    if (2 * std::min(nx, nz) > sms || t.nin > kLnMaxIn) return 0;
+    const size_t blk = (size_t)t.nface * t.nin * es, rest = (size_t)kLnBufs * (t.nin + t.nface) * sizeof(float);
+    const int ns = (int)std::min<size_t>(kLnStages, (kSwSmemMax - rest) / blk);
+    return ns >= 2 ? ns : 0;
+}
+
+template <typename AT, int NP>
+cudaError_t launch_lines(cudaLaunchConfig_t cfg, const SweepArgs& a, const void* A) {
+    const cudaError_t e = allow_smem(k_sweep_lines<AT, NP>);
+    if (e != cudaSuccess) return e;
+    cfg.gridDim = dim3(2u * (unsigned)std::min(a.nx, a.nz));
+    cfg.blockDim = dim3(32 * (ln_warps(a.nface) + kLnBufs + 1));
+    cfg.dynamicSmemBytes = (size_t)a.stages * a.nface * a.nin * sizeof(AT) + (size_t)kLnBufs * (a.nin + a.nface) * sizeof(float);
+    return cudaLaunchKernelEx(&cfg, k_sweep_lines<AT, NP>, a, (const AT*)A);
+}
+
 template <typename AT, int NP>
 cudaError_t launch_sweep(cudaLaunchConfig_t cfg, const SweepArgs& a, const void* A) {
     const size_t smem = (size_t)a.stages * a.nface * 2 * a.nin * sizeof(AT) + (((a.nin + 3) & ~3) + 32) * sizeof(float);
@@ -349,8 +633,11 @@ void sweep_orders(int nx, int nz, int* out) {
 // device scratch of one application's outflow words: four slots of E x n_in / 2 64-bit words
 size_t sweep_words_bytes(const Tab& t, int64_t E) { return (size_t)4 * E * (t.nin / 2) * sizeof(VerVal); }
 
+// whether an application on this mesh needs the item order (k_sweep), with operators of 4-byte entries
+bool sweep_needs_order(const Tab& t, int nx, int nz, int sms) { return line_stages(t, nx, nz, 4, sms) == 0; }
+
 // z = M u on the stream, with the operator A (FP16 or FP32, [E][nin][nin], 16-byte aligned);
-// order: device [4 E] from sweep_orders; zw: device scratch of sweep_words_bytes; flags: device ints
+// order: device [4 E] from sweep_orders (not read where sweep_needs_order says no); zw: device scratch of sweep_words_bytes; flags: device ints
 // (err, abort), cleared here (err stays set after a timed-out wait); z is zeroed first, so a skipped
 // application leaves 0.
 elrt_status sweep_apply(elrt_ctx* ctx, int nx, int nz, const void* A, int a_bytes, const float* u, float* z,
@@ -384,7 +671,15 @@ elrt_status sweep_apply(elrt_ctx* ctx, int nx, int nz, const void* A, int a_byte
     cfg.numAttrs = 1;
     const int npair = t.nin / 2;
     cudaError_t e;
-    if (npair <= 32 * 4)
+    if (const int ls = line_stages(t, nx, nz, a_bytes, nsm)) {
+        a.stages = ls;
+        if (npair <= 32 * 3)
+            e = a_bytes == 2 ? launch_lines<__half, 3>(cfg, a, A) : launch_lines<float, 3>(cfg, a, A);
+        else if (npair <= 32 * 4)
+            e = a_bytes == 2 ? launch_lines<__half, 4>(cfg, a, A) : launch_lines<float, 4>(cfg, a, A);
+        else
+            e = a_bytes == 2 ? launch_lines<__half, 5>(cfg, a, A) : launch_lines<float, 5>(cfg, a, A);
+    } else if (npair <= 32 * 4)
         e = a_bytes == 2 ? launch_sweep<__half, 4>(cfg, a, A) : launch_sweep<float, 4>(cfg, a, A);
     else if (npair <= 32 * 8)
         e = a_bytes == 2 ? launch_sweep<__half, 8>(cfg, a, A) : launch_sweep<float, 8>(cfg, a, A);
@@ -408,11 +703,13 @@ extern "C" elrt_status elrt_apply_precond(elrt_ctx* ctx, int32_t nx, int32_t nz,
     void* zw = ctx->vec;
     int* order = (int*)((unsigned char*)ctx->vec + wbytes);
     int* flags = order + 4 * E;
-    std::vector<int> ord((size_t)4 * E);
-    sweep_orders(nx, nz, ord.data());
-    s = cuda_check(ctx, cudaMemcpyAsync(order, ord.data(), ord.size() * sizeof(int), cudaMemcpyHostToDevice, ctx->stream),
-                   "sweep orders");
-    if (!s) s = cuda_check(ctx, cudaStreamSynchronize(ctx->stream), "sweep orders");
+    if (sweep_needs_order(ctx->tab, nx, nz, ctx->sms)) {
+        std::vector<int> ord((size_t)4 * E);
+        sweep_orders(nx, nz, ord.data());
+        s = cuda_check(ctx, cudaMemcpyAsync(order, ord.data(), ord.size() * sizeof(int), cudaMemcpyHostToDevice, ctx->stream),
+                       "sweep orders");
+        if (!s) s = cuda_check(ctx, cudaStreamSynchronize(ctx->stream), "sweep orders");
+    }
     if (!s) s = sweep_apply(ctx, nx, nz, in2out, 4, r, z, order, zw, flags, nullptr, nullptr);
     if (s) return s;
     int h = 0;
