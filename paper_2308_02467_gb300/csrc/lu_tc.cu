@@ -9,7 +9,7 @@
 // factored in panels of 64 columns, taken in pairs a = [J, J+64), b = [J+64, J+128):
 //   k_diag             (one small block per element): LU of the 64 x 64 diagonal block, published
 //                      as U11, L11^T, U11^T and 1 / diag(U11);
-//   k_rowcol           (blocks of 128 rows or columns per element): L21 from L21 U11 = A21 written
+//   k_rowcol           (blocks of 96 rows or 128 columns of an element): L21 from L21 U11 = A21 written
 //                      back to the matrix; U12 from L11 U12 = A12 written back to the matrix and,
 //                      transposed (K-major), to one side buffer whose rows hold both panels of the
 //                      pair as FP32 values and their low TF32 parts, or four panels as FP16 high parts
@@ -148,64 +148,76 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag(int nu, int64_t ld, int64
     rd[c] = 1.f / D[c][c];
 }
 
-// Triangular solves of one row or column held in registers, with the factor in shared memory
-// (row stride TI) and the reciprocal diagonal rd:
+// pairs of FP32 values in one 64-bit register, and the packed multiply-add on both (each half rounded as fmaf)
+using f2 = unsigned long long;
+__device__ __forceinline__ f2 f2_pack(float lo, float hi) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void f2_unpack(f2 v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
+    f2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+// Triangular solves of one row or column held in registers (a[m]: unknowns 2 m and 2 m + 1), with the factor
+// in shared memory (row stride TI) and the reciprocal diagonal rd:
 //   SolveKind 0 (row of L21):  x U = a     ->  x_i = a_i / U_ii, a_j -= x_i U[i][j] for j > i
 //   SolveKind 1 (forward):     L y = a     ->  y_i = a_i,        a_j -= LT[i][j] y_i for j > i
 //   SolveKind 2 (backward):    U y = a     ->  y_i = a_i / U_ii, a_j -= UT[i][j] y_i for j < i
 // (right-looking: every step updates independent accumulators).  Each finished 4-wide block of the
 // result is handed to put(b, float4): ascending b for kinds 0 and 1, descending for kind 2.
+// The unrolled solve is 3400 instructions a warp and stalls most on fetching them (issue slots 49 % used, HBM at
+// 24 %), so the updates are packed f32x2 multiply-adds: the same arithmetic and rate per value, half the
+// instructions.  Panel solves of 4096 elements (p = 6, N = 16): 14.0 ms with scalar ones, 12.8 packed.
 template <int SolveKind, typename Put>
-__device__ __forceinline__ void tri_solve(float (&a)[NBP], const float* __restrict__ T, const float* __restrict__ rd,
+__device__ __forceinline__ void tri_solve(f2 (&a)[NBP / 2], const float* __restrict__ T, const float* __restrict__ rd,
                                           Put put) {
-    if constexpr (SolveKind != 2) {
+    constexpr bool DN = SolveKind == 2;
 #pragma unroll
-        for (int b = 0; b < NBP / 4; ++b) {
-            float y[4];
+    for (int bb = 0; bb < NBP / 4; ++bb) {
+        const int b = DN ? NBP / 4 - 1 - bb : bb;
+        float y[4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int i = 4 * b + q;
-                const float x = SolveKind == 0 ? a[i] * rd[i] : a[i];
-                y[q] = x;
-                const float* Ti = T + i * TI;
-                const int j0 = (i + 4) & ~3;  // scalars up to the next 16-byte boundary, then float4
-#pragma unroll
-                for (int j = i + 1; j < j0; ++j) a[j] = fmaf(-x, Ti[j], a[j]);
-#pragma unroll
-                for (int j = j0; j < NBP; j += 4) {
-                    const float4 u = *reinterpret_cast<const float4*>(Ti + j);
-                    a[j] = fmaf(-x, u.x, a[j]);
-                    a[j + 1] = fmaf(-x, u.y, a[j + 1]);
-                    a[j + 2] = fmaf(-x, u.z, a[j + 2]);
-                    a[j + 3] = fmaf(-x, u.w, a[j + 3]);
+        for (int qq = 0; qq < 4; ++qq) {
+            const int q = DN ? 3 - qq : qq, i = 4 * b + q, m = i >> 1;
+            float lo, hi;
+            f2_unpack(a[m], lo, hi);
+            const float v = i & 1 ? hi : lo;
+            const float x = SolveKind == 1 ? v : v * rd[i];
+            y[q] = x;
+            const f2 nx = f2_pack(-x, -x);
+            const float* Ti = T + i * TI;
+            // the rest of this block of four: the other half of the pair, and the other pair
+            if (!DN ? q == 0 : q == 3) {
+                const float4 u = *reinterpret_cast<const float4*>(Ti + 4 * b);
+                if (!DN) {
+                    a[m] = f2_pack(lo, fmaf(-x, u.y, hi));
+                    a[m + 1] = f2_fma(nx, f2_pack(u.z, u.w), a[m + 1]);
+                } else {
+                    a[m] = f2_pack(fmaf(-x, u.z, lo), hi);
+                    a[m - 1] = f2_fma(nx, f2_pack(u.x, u.y), a[m - 1]);
                 }
+            } else if (!DN ? q == 1 : q == 2) {
+                const int o = DN ? m - 1 : m + 1;
+                a[o] = f2_fma(nx, *reinterpret_cast<const f2*>(Ti + 2 * o), a[o]);
+            } else if (!DN && q == 2) {
+                a[m] = f2_pack(lo, fmaf(-x, Ti[i + 1], hi));
+            } else if (DN && q == 1) {
+                a[m] = f2_pack(fmaf(-x, Ti[i - 1], lo), hi);
             }
-            put(b, make_float4(y[0], y[1], y[2], y[3]));
-        }
-    } else {
+            // the blocks beyond
 #pragma unroll
-        for (int b = NBP / 4 - 1; b >= 0; --b) {
-            float y[4];
-#pragma unroll
-            for (int q = 3; q >= 0; --q) {
-                const int i = 4 * b + q;
-                const float x = a[i] * rd[i];
-                y[q] = x;
-                const float* Ti = T + i * TI;
-                const int j1 = i & ~3;  // float4 below the 16-byte boundary, then scalars
-#pragma unroll
-                for (int j = 0; j < j1; j += 4) {
-                    const float4 u = *reinterpret_cast<const float4*>(Ti + j);
-                    a[j] = fmaf(-x, u.x, a[j]);
-                    a[j + 1] = fmaf(-x, u.y, a[j + 1]);
-                    a[j + 2] = fmaf(-x, u.z, a[j + 2]);
-                    a[j + 3] = fmaf(-x, u.w, a[j + 3]);
-                }
-#pragma unroll
-                for (int j = j1; j < i; ++j) a[j] = fmaf(-x, Ti[j], a[j]);
+            for (int c = 0; c < NBP / 4; ++c) {
+                if (DN ? c >= b : c <= b) continue;
+                const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(Ti + 4 * c);
+                a[2 * c] = f2_fma(nx, u.x, a[2 * c]);
+                a[2 * c + 1] = f2_fma(nx, u.y, a[2 * c + 1]);
             }
-            put(b, make_float4(y[0], y[1], y[2], y[3]));
         }
+        put(b, make_float4(y[0], y[1], y[2], y[3]));
     }
 }
 
@@ -215,8 +227,8 @@ __device__ __forceinline__ void tri_solve(float (&a)[NBP], const float* __restri
 // c_end): y = L11^{-1} a (col_mode 0: factorisation and forward sweep) or y = U11^{-1} a
 // (col_mode 1: backward sweep), written back to the matrix (rows < jb) and, transposed, to the side
 // buffer Ut[e][column][koff .. koff + 63] (zero beyond jb), with its low TF32 parts at K offset
-// UTL + koff.  Persistent, four blocks of 128 threads per SM (one staging buffer each, 128
-// registers per thread): each block walks its items, copying an item's 64-wide block and the factor
+// UTL + koff.  Persistent, four or five blocks of one thread per row or column per SM (one staging buffer
+// each, 128 registers per thread): each block walks its items, copying an item's 64-wide block and the factor
 // of the diagonal block with 16-byte cp.async copies, solving and storing it; the blocks of an SM
 // overlap one another's copies and stores.  (One block per SM with two staging buffers, copies of
 // the next item in flight, measured 23% slower: 8 warps per SM were too few to hide the
@@ -227,12 +239,15 @@ template <int PTILE>
 struct RcCfg {
     static constexpr int BUF = PTILE * RS + (NBP + 1) * RS;  // floats: staging + factor + 1/diag
     static constexpr int SMEM = BUF * (int)sizeof(float);
-    static constexpr int PER_SM = PTILE == 256 ? 2 : 4;      // resident blocks per SM
+    static constexpr int PER_SM = PTILE == 96 ? 5 : 4;       // resident blocks per SM
     static_assert(PTILE * RS >= NBP * PTILE, "the staging area holds a 64 x PTILE column block");
 };
-// 128-row tiles, four blocks per SM: measured 2 % faster than 256-row tiles with two blocks per SM
-// (the same 16 warps, more independent copy / solve / store phases to overlap)
-constexpr int kRcTile = 128;
+// Smaller tiles leave more independent copy / solve / store phases on an SM to overlap, larger ones copy the
+// factor less often.  In the 4096-element build with p = 6, N = 16: rows in tiles of 96, five blocks per SM,
+// 3.13 ms, 128 with four blocks 3.28; columns (wider staging per solve, and their results stored twice)
+// 96 10.7 ms, 128 9.5 (256 with two blocks 2 % more).  Columns read straight into registers while the item
+// before is stored, instead of staged, 11.2.
+constexpr int kRowTile = 96, kColTile = 128;
 
 __device__ __forceinline__ void cp_async16(float* smem, const float* gmem, bool valid) {
     // src-size 0 fills the 16 bytes with zeros and reads nothing
@@ -316,9 +331,9 @@ __global__ void __launch_bounds__(PTILE, RcCfg<PTILE>::PER_SM) k_rowcol(int nu, 
         if constexpr (KIND == 0) {
             const int r0 = r_begin + tile * PTILE, nr = min(PTILE, r_end - r0);
             if (t < nr) {  // x U11 = a, written over the row it came from
-                float a[NBP];
+                f2 a[NBP / 2];
 #pragma unroll
-                for (int i = 0; i < NBP; ++i) a[i] = S[t * RS + i];
+                for (int i = 0; i < NBP / 2; ++i) a[i] = *reinterpret_cast<const f2*>(S + t * RS + 2 * i);
                 float* out = S + t * RS;
                 tri_solve<0>(a, T, T + NBP * RS, [&](int bb, float4 v) { *reinterpret_cast<float4*>(out + 4 * bb) = v; });
             }
@@ -337,10 +352,10 @@ __global__ void __launch_bounds__(PTILE, RcCfg<PTILE>::PER_SM) k_rowcol(int nu, 
             }
         } else if constexpr (KIND != 0) {
             const int c0 = c_begin + (tile - nrt) * PTILE, nc = min(PTILE, c_end - c0);
-            float a[NBP];
+            f2 a[NBP / 2];
             if (t < nc) {
 #pragma unroll
-                for (int k = 0; k < NBP; ++k) a[k] = S[k * PTILE + t];
+                for (int k = 0; k < NBP / 2; ++k) a[k] = f2_pack(S[2 * k * PTILE + t], S[(2 * k + 1) * PTILE + t]);
             }
             __syncthreads();  // S is reused: from [k][column] staging to [column][i] results
             if (t < nc) {
@@ -945,14 +960,6 @@ elrt_status update(elrt_ctx* ctx, const TcMaps& mp, float* M, int64_t ld, int64_
 }
 
 
-template <int PT>
-cudaError_t rowcol_attrs() {
-    cudaError_t e = cudaFuncSetAttribute(k_rowcol<0, PT>, cudaFuncAttributeMaxDynamicSharedMemorySize, RcCfg<PT>::SMEM);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_rowcol<1, PT>, cudaFuncAttributeMaxDynamicSharedMemorySize, RcCfg<PT>::SMEM);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_rowcol<2, PT>, cudaFuncAttributeMaxDynamicSharedMemorySize, RcCfg<PT>::SMEM);
-    return e;
-}
-
 elrt_status prepare(elrt_ctx* ctx, float* M, int64_t ld, int64_t estride, const float* Ut, int64_t E, TcMaps* mp,
                     bool f16) {
     mp->f16 = f16;
@@ -966,7 +973,12 @@ elrt_status prepare(elrt_ctx* ctx, float* M, int64_t ld, int64_t estride, const 
         return ctx_fail(ctx, ELRT_EINVAL, "tensor map encoding failed");
     static bool attr_done = false;
     if (!attr_done) {
-        cudaError_t e = rowcol_attrs<kRcTile>();
+        cudaError_t e = cudaFuncSetAttribute(k_rowcol<0, kRowTile>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             RcCfg<kRowTile>::SMEM);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_rowcol<1, kColTile>, cudaFuncAttributeMaxDynamicSharedMemorySize, RcCfg<kColTile>::SMEM);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_rowcol<2, kColTile>, cudaFuncAttributeMaxDynamicSharedMemorySize, RcCfg<kColTile>::SMEM);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_tc_update<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, UpdCfg<64>::TOTAL);
         if (e == cudaSuccess)
@@ -988,30 +1000,6 @@ elrt_status prepare(elrt_ctx* ctx, float* M, int64_t ld, int64_t estride, const 
 
 int panels_of(int nu) { return (nu + NBP - 1) / NBP; }
 
-template <int PTILE>
-void rowcol_launch(elrt_ctx* ctx, float* M, int64_t ld, int64_t estride, int64_t E, int J, int jb, const float* Tinv,
-                   int r_begin, int r_end, int c_begin, int c_end, int col_mode, float* Ut, int koff, int ut16,
-                   const double* res_max) {
-    using C = RcCfg<PTILE>;
-    const int nrt = r_end > r_begin ? (r_end - r_begin + PTILE - 1) / PTILE : 0;
-    const int nct = c_end > c_begin ? (c_end - c_begin + PTILE - 1) / PTILE : 0;
-    const int np = panels_of(ctx->tab.nu), nu = ctx->tab.nu;
-    if (nrt > 0) {  // items: (element, row tile)
-        const unsigned grid = (unsigned)std::min<int64_t>(E * nrt, (int64_t)C::PER_SM * ctx->sms);
-        k_rowcol<0, PTILE><<<grid, PTILE, C::SMEM, ctx->stream>>>(nu, ld, estride, M, J, jb, Tinv, np, E, r_begin, r_end,
-                                                                 nrt, c_begin, c_end, 0, Ut, koff, ut16, nullptr);
-    }
-    if (nct > 0) {  // items: (element, column tile)
-        const unsigned grid = (unsigned)std::min<int64_t>(E * nct, (int64_t)C::PER_SM * ctx->sms);
-        if (col_mode == 0)
-            k_rowcol<1, PTILE><<<grid, PTILE, C::SMEM, ctx->stream>>>(nu, ld, estride, M, J, jb, Tinv, np, E, r_begin,
-                                                                     r_end, 0, c_begin, c_end, nct, Ut, koff, ut16, res_max);
-        else
-            k_rowcol<2, PTILE><<<grid, PTILE, C::SMEM, ctx->stream>>>(nu, ld, estride, M, J, jb, Tinv, np, E, r_begin,
-                                                                     r_end, 0, c_begin, c_end, nct, Ut, koff, ut16, nullptr);
-    }
-}
-
 elrt_status rowcol(elrt_ctx* ctx, const TcMaps& mp, float* M, int64_t ld, int64_t estride, int64_t E, int J, int jb,
                    const float* Tinv, int r_begin, int r_end, int c_begin, int c_end, int col_mode, float* Ut,
                    int koff = 0) {
@@ -1022,8 +1010,23 @@ elrt_status rowcol(elrt_ctx* ctx, const TcMaps& mp, float* M, int64_t ld, int64_
     const double bytes = 8.0 * R * jb + 8.0 * C * jb + 4.0 * C * NBP + 4.0 * NBP * NBP * ((R > 0) + (C > 0));
     const double flops = R * jb * (jb + 1.0) + (col_mode == 0 ? C * jb * (jb - 1.0) : C * jb * (jb + 1.0));
     ProfScope ps(ctx, "lu_tc_rowcol", (R > 0) + (C > 0), (double)E * bytes, (double)E * flops);
-    rowcol_launch<kRcTile>(ctx, M, ld, estride, E, J, jb, Tinv, r_begin, r_end, c_begin, c_end, col_mode, Ut, koff,
-                           mp.f16 ? 1 : 0, mp.res_max);
+    const int np = panels_of(ctx->tab.nu), nu = ctx->tab.nu, ut16 = mp.f16 ? 1 : 0;
+    const auto launch = [&](auto kern, int tile, int per_sm, int smem, int nrt, int nct, const double* rmax) {
+        const unsigned grid = (unsigned)std::min<int64_t>(E * (nrt + nct), (int64_t)per_sm * ctx->sms);
+        kern<<<grid, tile, smem, ctx->stream>>>(nu, ld, estride, M, J, jb, Tinv, np, E, r_begin, r_end, nrt, c_begin,
+                                                c_end, nct, Ut, koff, ut16, rmax);
+    };
+    using Cr = RcCfg<kRowTile>;
+    using Cc = RcCfg<kColTile>;
+    if (r_end > r_begin)
+        launch(k_rowcol<0, kRowTile>, kRowTile, Cr::PER_SM, Cr::SMEM, (r_end - r_begin + kRowTile - 1) / kRowTile, 0, nullptr);
+    if (c_end > c_begin) {
+        const int nct = (c_end - c_begin + kColTile - 1) / kColTile;
+        if (col_mode == 0)
+            launch(k_rowcol<1, kColTile>, kColTile, Cc::PER_SM, Cc::SMEM, 0, nct, mp.res_max);
+        else
+            launch(k_rowcol<2, kColTile>, kColTile, Cc::PER_SM, Cc::SMEM, 0, nct, nullptr);
+    }
     return cuda_check(ctx, cudaGetLastError(), "rowcol launch");
 }
 
