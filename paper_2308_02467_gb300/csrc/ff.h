@@ -79,6 +79,72 @@ __device__ __forceinline__ void ff_fma_f(ff& acc, float a, ff x) {
     acc.l = __fadd_rn(acc.l, __fadd_rn(t, e));
 }
 
+// Two FP32 values in one 64-bit register, and the packed operations: each half is rounded as the scalar
+// operation rounds it, at the same rate per value, for half the instructions.
+using f2 = unsigned long long;
+__device__ __forceinline__ f2 f2_pack(float lo, float hi) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void f2_unpack(f2 v, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
+    f2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
+    f2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f2 f2_add(f2 a, f2 b) {
+    f2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f2 f2_sub(f2 a, f2 b) {
+    f2 d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+// two float-float accumulators side by side, the low parts negated (the packed multiply-add takes no negated
+// operand: with -c beside c the product's error comes out negated), and a pair of coefficients for them
+struct ff2 {
+    f2 h, nl;
+};
+struct ffc2 {
+    f2 h, nh, nl;  // c.h, -c.h, -c.l
+};
+
+// acc = c (xh + xl) and acc += c (xh + xl): ff_fma on both halves, the same roundings
+__device__ __forceinline__ ff2 ff2_mul0(const ffc2& c, f2 xh, f2 xl) {
+    const f2 p = f2_mul(c.h, xh);
+    f2 e = f2_fma(c.nh, xh, p);
+    e = f2_fma(c.nh, xl, e);
+    return ff2{p, f2_fma(c.nl, xh, e)};
+}
+__device__ __forceinline__ void ff2_fma(ff2& acc, const ffc2& c, f2 xh, f2 xl) {
+    const f2 p = f2_mul(c.h, xh);
+    f2 e = f2_fma(c.nh, xh, p);
+    e = f2_fma(c.nh, xl, e);
+    e = f2_fma(c.nl, xh, e);
+    const f2 s = f2_add(acc.h, p), bp = f2_sub(s, acc.h);
+    const f2 nt = f2_add(f2_sub(f2_sub(s, bp), acc.h), f2_sub(bp, p));
+    acc.h = s;
+    acc.nl = f2_add(acc.nl, f2_add(nt, e));
+}
+__device__ __forceinline__ void ff2_split(const ff2& v, ff& a, ff& b) {
+    float la, lb;
+    f2_unpack(v.h, a.h, b.h);
+    f2_unpack(v.nl, la, lb);
+    a.l = -la;
+    b.l = -lb;
+}
+
 // warp-wide sum of (h, l) pairs; the result is valid in lane 0
 __device__ __forceinline__ ff ff_warp_sum(ff a) {
 #pragma unroll

@@ -44,6 +44,7 @@
 #include <cudaTypedefs.h>
 
 #include "elrt_internal.h"
+#include "ff.h"
 #include "tc_gemm.cuh"
 
 namespace {
@@ -146,20 +147,6 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag(int nu, int64_t ld, int64
         UT[idx] = cc <= r ? D[cc][r] : 0.f;   // UT[r][c] = U[c][r]
     }
     rd[c] = 1.f / D[c][c];
-}
-
-// pairs of FP32 values in one 64-bit register, and the packed multiply-add on both (each half rounded as fmaf)
-using f2 = unsigned long long;
-__device__ __forceinline__ f2 f2_pack(float lo, float hi) {
-    f2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void f2_unpack(f2 v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
-__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
-    f2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
 }
 
 // Triangular solves of one row or column held in registers (a[m]: unknowns 2 m and 2 m + 1), with the factor

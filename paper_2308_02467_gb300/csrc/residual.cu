@@ -1,10 +1,9 @@
 // Float-float refinement residual of the FP32 / TF32 local solves for the common element shapes:
 // R = -B^ - A X from the structured operator (eq. hdg_local_mat), with X kept as float-float pairs.
 //
-// What bounds it: the FP32 pipes.  A float-float multiply-add is 11 or 12 FP32 instructions, and GB300
-// issues 39.8e12 scalar FP32 lane operations a second (measured; packed f32x2 instructions reach the same
-// rate), so the kernel's time is its instruction count.  Two symmetries of the operator halve the
-// multiply-adds:
+// What bounds it: the FP32 pipes.  A float-float multiply-add is 11 or 12 FP32 operations, and GB300
+// carries out 39.8e12 FP32 lane operations a second, in scalar or packed f32x2 instructions (measured).  Two
+// symmetries of the operator halve the multiply-adds:
 //   * the phase matrix is circulant, W[k][l] = wc[(k - l) mod N]: with H = N / 2 and the sums and
 //     differences p_l = x_l + x_{l+H}, m_l = x_l - x_{l+H}, the angular sum of all N directions is two
 //     H x H products (S_k = sum cp[k-l] p_l, D_k = sum cm[k-l] m_l; y_k = S_k + D_k, y_{k+H} = S_k - D_k),
@@ -18,10 +17,15 @@
 // scattering, x-lines, z-lines with the final residual -- accumulating in float-float.  Eight columns
 // (32-byte sectors of a row) leave room for two blocks per SM at p = 6, N = 16, so one block's copies
 // and barriers overlap the other's arithmetic; the next chunk's columns arrive by cp.async meanwhile.
+// The two halves of each split run side by side in packed f32x2 instructions, half the instructions for the
+// same roundings (ff2_fma): with scalar ones the issue slots were 70 % used and the pipe 61 %; now waiting for
+// the pipe is the first stall.
 // Measured against the general kernel of local.cu (one row and two columns per thread, every sum in full):
-// 4096 elements at p = 6, N = 16, first pass, 11.2 -> 7.6 ms; 1247 elements at p = 8, N = 16, 9.7 -> 6.2 ms
-// for the first and 12.1 -> 7.5 ms for a later pass.
+// 4096 elements at p = 6, N = 16, adjoint form, 11.2 -> 7.5 ms, packed 6.85 ms; 1247 elements at p = 8, N = 16,
+// 9.7 -> 5.6 ms for the first and 12.1 -> 7.2 ms for a later pass; 480 elements at p = 6, N = 16, first pass,
+// 0.86 ms.
 #include <algorithm>
+#include <cstring>
 
 #include "elrt_internal.h"
 #include "ff.h"
@@ -32,9 +36,11 @@ constexpr int kCW = 8;  // columns per pass
 
 // Coefficients of the split sums, as float-float pairs (constant bank)
 struct ResTab {
-    ff cp[ELRT_MAX_ANG / 2], cm[ELRT_MAX_ANG / 2];  // (wc[d] + wc[d + H]) / 2, (wc[d] - wc[d + H]) / 2, d < H
-    ff U[5 * 5];  // [a][q] (wd[q][a] - wd[p-q][a]) / 2: coefficients of the differences o_q
-    ff V[5 * 6];  // [a][q] (wd[q][a] + wd[p-q][a]) / 2: of the sums e_q; q = h: wd[h][a], of the middle node
+    // d < H: (wc[d] + wc[d + H]) / 2 beside (wc[d] - wc[d + H]) / 2; d + H: the same, the second one negated
+    ffc2 W[ELRT_MAX_ANG];
+    // [a][q] (wd[q][a] - wd[p-q][a]) / 2, of the difference o_q, beside (wd[q][a] + wd[p-q][a]) / 2, of the sum e_q
+    ffc2 UV[5 * 5];
+    ff V[5];      // wd[h][a], of the middle node
     ff mid[5];    // wd[q][h]: the middle output takes the differences only
 };
 
@@ -64,20 +70,20 @@ __device__ __forceinline__ ff neg(ff a) { return ff{-a.h, -a.l}; }
 template <int N, typename XS, typename Put>
 __device__ __forceinline__ void angular(const ResTab& rt, const XS (&x)[N], Put put) {
     constexpr int H = N / 2;
-    ff p[H], m[H];
+    f2 xh[H], xl[H];  // (sum, difference)
 #pragma unroll
     for (int l = 0; l < H; ++l) {
-        p[l] = sum2(x[l], x[l + H]);
-        m[l] = sum2(x[l], neg(x[l + H]));
+        const ff p = sum2(x[l], x[l + H]), m = sum2(x[l], neg(x[l + H]));
+        xh[l] = f2_pack(p.h, m.h);
+        xl[l] = f2_pack(p.l, m.l);
     }
 #pragma unroll
     for (int k = 0; k < H; ++k) {
-        ff s = mul0(rt.cp[k], p[0]), d = mul0(rt.cm[k], m[0]);
+        ff2 sd = ff2_mul0(rt.W[k], xh[0], xl[0]);
 #pragma unroll
-        for (int l = 1; l < H; ++l) {
-            mac(s, rt.cp[(k - l + H) % H], p[l]);
-            mac(d, rt.cm[(k - l + H) % H], k >= l ? m[l] : neg(m[l]));  // cm[d + H] = -cm[d]
-        }
+        for (int l = 1; l < H; ++l) ff2_fma(sd, rt.W[k >= l ? k - l : k - l + 2 * H], xh[l], xl[l]);  // cm[d + H] = -cm[d]
+        ff s, d;
+        ff2_split(sd, s, d);
         put(k, ff_add(s, d));
         put(k + H, ff_add(s, neg(d)));
     }
@@ -87,21 +93,23 @@ __device__ __forceinline__ void angular(const ResTab& rt, const XS (&x)[N], Put 
 template <int N1, typename XS, typename Put>
 __device__ __forceinline__ void line(const ResTab& rt, const XS (&x)[N1], Put put) {
     constexpr int h = N1 / 2;
-    ff e[h], o[h];
+    f2 xh[h], xl[h];  // (difference, sum)
+    ff o[h];
 #pragma unroll
     for (int q = 0; q < h; ++q) {
-        e[q] = sum2(x[q], x[N1 - 1 - q]);
+        const ff e = sum2(x[q], x[N1 - 1 - q]);
         o[q] = sum2(x[q], neg(x[N1 - 1 - q]));
+        xh[q] = f2_pack(o[q].h, e.h);
+        xl[q] = f2_pack(o[q].l, e.l);
     }
 #pragma unroll
     for (int a = 0; a < h; ++a) {
-        ff u = mul0(rt.U[a * 5], o[0]), v = mul0(rt.V[a * 6], e[0]);
+        ff2 uv = ff2_mul0(rt.UV[a * 5], xh[0], xl[0]);
 #pragma unroll
-        for (int q = 1; q < h; ++q) {
-            mac(u, rt.U[a * 5 + q], o[q]);
-            mac(v, rt.V[a * 6 + q], e[q]);
-        }
-        mac(v, rt.V[a * 6 + h], x[h]);
+        for (int q = 1; q < h; ++q) ff2_fma(uv, rt.UV[a * 5 + q], xh[q], xl[q]);
+        ff u, v;
+        ff2_split(uv, u, v);
+        mac(v, rt.V[a], x[h]);
         put(a, ff_add(u, v));
         put(N1 - 1 - a, ff_add(u, neg(v)));
     }
@@ -156,7 +164,9 @@ __global__ void __launch_bounds__(ResCfg<N1, N, XS>::T, ResCfg<N1, N, XS>::BLOCK
     ff* X = Xall + e * (int64_t)(ADJ ? NM : NU) * nin;
     float* Rp = ADJ ? Rall + e * (int64_t)NU * nin : M;
     const int64_t rld = ADJ ? nin : ld;
-    const int step = gridDim.y * kCW;
+    // this block's columns: neighbouring chunks, whose rows share cache lines
+    const int per = (nin / kCW + gridDim.y - 1) / gridDim.y * kCW;
+    const int cs0 = min(nin, (int)blockIdx.y * per), cs1 = min(nin, cs0 + per);
     auto prefetch = [&](int cs, XS* dst) {  // first pass: the chunk's columns of D (two 16-byte halves a row)
         if constexpr (F) {
             for (int q = tid; q < 2 * NU; q += T)
@@ -164,7 +174,7 @@ __global__ void __launch_bounds__(ResCfg<N1, N, XS>::T, ResCfg<N1, N, XS>::BLOCK
             asm volatile("cp.async.commit_group;" ::: "memory");
         }
     };
-    prefetch(blockIdx.y * kCW, Xs);
+    if (cs0 < cs1) prefetch(cs0, Xs);
     const double he = h_elem ? h_elem[e] : h;
     const double om = omega[e];
     for (int q = tid; q < NM; q += T)
@@ -187,13 +197,13 @@ __global__ void __launch_bounds__(ResCfg<N1, N, XS>::T, ResCfg<N1, N, XS>::BLOCK
     const int col = tid & (kCW - 1), g = tid / kCW;
     float rmax = 0.f;
     int buf = 0;
-    for (int cs = blockIdx.y * kCW; cs < nin; cs += step, buf ^= 1) {
+    for (int cs = cs0; cs < cs1; cs += kCW, buf ^= 1) {
         const XS* xs = Xs;
         if constexpr (F) {
             asm volatile("cp.async.wait_all;" ::: "memory");
             __syncthreads();  // the chunk has landed; the last pass over the other buffer is done
             xs = Xs + (size_t)buf * NU * kCW;
-            if (cs + step < nin) prefetch(cs + step, Xs + (size_t)(buf ^ 1) * NU * kCW);
+            if (cs + kCW < cs1) prefetch(cs + kCW, Xs + (size_t)(buf ^ 1) * NU * kCW);
             if constexpr (!ADJ)
                 for (int r = g; r < NU; r += G) X[(int64_t)r * nin + cs + col] = ff{xs[r * kCW + col], 0.f};
         } else {
@@ -299,17 +309,26 @@ __global__ void __launch_bounds__(ResCfg<N1, N, XS>::T, ResCfg<N1, N, XS>::BLOCK
 ResTab make_tab(const Tab& t) {
     ResTab r{};
     const int H = t.N / 2, n1 = t.n1, h = n1 / 2;
+    auto pair = [](double a, double b) {
+        const ff x = ff_from_double_host(a), y = ff_from_double_host(b);
+        auto two = [](float lo, float hi) {
+            const float v[2] = {lo, hi};
+            f2 r;
+            memcpy(&r, v, sizeof(r));
+            return r;
+        };
+        return ffc2{two(x.h, y.h), two(-x.h, -y.h), two(-x.l, -y.l)};
+    };
     for (int d = 0; d < H; ++d) {
-        r.cp[d] = ff_from_double_host(0.5 * (t.wc[d] + t.wc[d + H]));
-        r.cm[d] = ff_from_double_host(0.5 * (t.wc[d] - t.wc[d + H]));
+        const double cp = 0.5 * (t.wc[d] + t.wc[d + H]), cm = 0.5 * (t.wc[d] - t.wc[d + H]);
+        r.W[d] = pair(cp, cm);
+        r.W[d + H] = pair(cp, -cm);
     }
     auto wd = [&](int q, int a) { return t.w[q] * t.D[q * n1 + a]; };
     for (int a = 0; a < h; ++a) {
-        for (int q = 0; q < h; ++q) {
-            r.U[a * 5 + q] = ff_from_double_host(0.5 * (wd(q, a) - wd(n1 - 1 - q, a)));
-            r.V[a * 6 + q] = ff_from_double_host(0.5 * (wd(q, a) + wd(n1 - 1 - q, a)));
-        }
-        r.V[a * 6 + h] = ff_from_double_host(wd(h, a));
+        for (int q = 0; q < h; ++q)
+            r.UV[a * 5 + q] = pair(0.5 * (wd(q, a) - wd(n1 - 1 - q, a)), 0.5 * (wd(q, a) + wd(n1 - 1 - q, a)));
+        r.V[a] = ff_from_double_host(wd(h, a));
         r.mid[a] = ff_from_double_host(wd(a, h));
     }
     return r;
@@ -333,9 +352,19 @@ elrt_status launch(const Args& a) {
     const Tab& t = a.ctx->tab;
     cudaError_t e = cudaFuncSetAttribute(k_residual_eo<N1, N, XS, ADJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
     if (e != cudaSuccess) return cuda_check(a.ctx, e, "smem attribute");
-    // a batch too small to fill the GPU spreads each element's column chunks over several blocks
-    const int64_t fit = (int64_t)Cfg::BLOCKS * a.ctx->sms / std::max<int64_t>(a.n, 1);
-    const int gy = (int)std::max<int64_t>(1, std::min<int64_t>(t.nin / kCW, fit));
+    // gy blocks share an element's column chunks: as many as make (waves of blocks) x (chunks a block takes,
+    // and half a one for its coefficients and its first load) least.  A small batch fills the GPU that way, and a
+    // larger one loses less to its last wave: against one block an element, 480 elements (p = 6, N = 16; gy = 5)
+    // 1.11 -> 0.86 ms, 1247 (p = 8; gy = 4) 6.18 -> 5.57 ms.  The blocks take neighbouring chunks: taken in turn,
+    // 0.94 and 5.87 ms, and the pass that reads X too 8.4 instead of 7.2 (its cache lines came in for each block).
+    const int64_t slots = (int64_t)Cfg::BLOCKS * a.ctx->sms;
+    const int chunks = t.nin / kCW;
+    int gy = 1;
+    int64_t least = INT64_MAX;
+    for (int y = 1; y <= chunks; ++y) {
+        const int64_t cost = ((a.n * y + slots - 1) / slots) * (2 * ((chunks + y - 1) / y) + 1);
+        if (cost < least) least = cost, gy = y;
+    }
     if (gy > 1 && !ADJ) {
         e = cudaMemsetAsync(a.maxres, 0, (size_t)a.n * sizeof(double), a.ctx->stream);
         if (e != cudaSuccess) return cuda_check(a.ctx, e, "residual maxima");

@@ -34,3 +34,24 @@ def test_refined_operators_of_every_shape(lib, p, N):
         for e in range(6):
             np.testing.assert_allclose(a[e::6].cpu().numpy(), np.broadcast_to(ops[e][0], (copies, *ops[e][0].shape)), atol=1e-10)
             np.testing.assert_allclose(m[e::6].cpu().numpy(), np.broadcast_to(ops[e][1], (copies, *ops[e][1].shape)), atol=1e-10)
+
+
+@pytest.mark.parametrize("p,N", [(2, 8), (4, 12), (6, 16), (8, 16)])
+@pytest.mark.parametrize("steps", [1, 2])
+def test_residual_does_not_depend_on_the_batch(lib, p, N, steps):
+    """However many blocks share an element's columns (a rule on the batch size), the arithmetic of a column is the
+    same: copies of one element come out with the bits of the element alone."""
+    import torch
+    k, o, _ = H.random_elements(1, p, seed=40 + p)
+    ctx = lib.Context(p, N, 0.85, lib.ANG_FV0)
+    first = None
+    for n in (1, 7, 77, 153, 305, 481):
+        a = torch.empty(n, ctx.nin, ctx.nin, dtype=torch.float64, device="cuda")
+        m = torch.empty(n, ctx.nm, ctx.nin, dtype=torch.float64, device="cuda")
+        kappa, omega = torch.tensor(np.repeat(k, n, 0), device="cuda"), torch.tensor(np.repeat(o, n), device="cuda")
+        st = ctx.elrt_build_local(kappa, omega, 0.3, a, m, mode=lib.LOCAL_TF32_IR, refine_steps=steps)
+        if first is None:
+            first = a[0].clone(), m[0].clone(), st.max_rel_residual
+        assert torch.equal(a, first[0].expand_as(a)) and torch.equal(m, first[1].expand_as(m))
+        assert st.max_rel_residual == first[2]
+    ctx.close()
