@@ -23,9 +23,9 @@
 // k_adjoint: one CTA per (element, tile of up to 128 of the n_in columns of r): D[j][c] = sum_rows r[row][j]
 // XZ[reversed row][c] in 3xTF32 on the tensor cores (FP32 values are their own high part; the full FP32 range,
 // so no scaling), j on the 128 lanes, c on up to 512 columns of tensor memory.  Both operands lie row-major
-// with the summation index outermost, so sixteen warps load them with 16-byte loads (four rows of four
+// with the summation index outermost, so fifteen warps load them with 16-byte loads (four rows of four
 // columns a lane), transpose in registers and write K-major, 128-byte-swizzled tiles of 32 rows of the sum,
-// eight lanes on one row's eight chunks (no bank conflicts); one thread of a seventeenth warp issues the MMAs.
+// eight lanes on one row's eight chunks (no bank conflicts); one thread of a sixteenth warp issues the MMAs.
 // Bound by the latency of its loads (about 2.4 MB per element in two column tiles, the second tile's mostly
 // from L2; DRAM 25 % and the tensor pipe 28 % busy): 16 warps and two stages of 106 KB are what one SM holds.  The epilogue reads X at the outflow rows, adds the correction
 // and rounds once.  Measured, builds with one refinement step: 4096 elements at p = 6, N = 16, 61.9 -> 51.6 ms
