@@ -128,10 +128,16 @@ elrt_status local_build(elrt_ctx* ctx, int64_t E, double h, const double* h_elem
                         const elrt_local_extras* extras = nullptr);
 
 // ---- tensor-core LU (lu_tc.cu).  f16: the trailing updates form their products as 3xFP16 (FP16
-// high parts and remainders, half the MMA instructions of 3xTF32), allowed for a factorisation when
-// every entry of the assembled matrices lies in [kLuF16Max / 4096, kLuF16Max]; the refinement
-// re-solves pass false (their right-hand sides are residuals far below FP16's normal range).
-constexpr float kLuF16Max = 1024.f;
+// high parts and remainders, half the MMA instructions of 3xTF32), allowed for a chunk when the
+// largest entry of its assembled matrices lies in [kLuF16Min, kLuF16Max].
+// The upper end leaves room for what the entries do not bound: the factors and solutions of thick elements
+// without absorption grow past FP16's 65504 before the entries do.  In exact arithmetic the solution of an
+// isotropic unit source (a right-hand side of the adjoint step) is up to 33 times the largest entry at p = 8
+// (albedo 1, g = 0, kappa inversely proportional to the quadrature weights) and L21 of a thick shell
+// around a thin core up to 12 times; the rounded factorisation of these nearly singular systems adds to it.
+// Measured, one-step builds of 1380 such elements, p = 2 .. 9: 18 elements not finite at a largest entry of
+// 1000 and 4 at 500, none at 250 and 125; at 250 the two forms are equally accurate.
+constexpr float kLuF16Min = 0.25f, kLuF16Max = 256.f;
 constexpr int kAsmMaxFlag = 24;  // d_flags slot: largest |entry| of the assembled FP32 matrices (float bits)
 elrt_status tc_lu_factor_solve(elrt_ctx* ctx, float* M, int64_t ld, int64_t estride, int64_t E, int* estat, float* side,
                                int* err, int nrhs, bool f16);

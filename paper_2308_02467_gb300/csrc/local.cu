@@ -1454,7 +1454,7 @@ elrt_status build_chunked(elrt_ctx* ctx, int64_t E, double h, const double* h_el
                                                                         estride, n);
         s = cuda_check(ctx, cudaGetLastError(), "assemble launch");
         if (s) return s;
-        // 3xFP16 trailing updates when every entry of the chunk's matrices lies in [kLuF16Max / 4096,
+        // 3xFP16 trailing updates when the largest entry of the chunk's matrices lies in [kLuF16Min,
         // kLuF16Max] (the entries are O(1): transport 0.5 at the boundary nodes, absorption w^2 kappa_hat)
         // and no source column rides along (its scale is the caller's); the refinement re-solves then
         // run their forward sweep in 3xFP16 too, each element's residual scaled by a power of two into
@@ -1469,7 +1469,7 @@ elrt_status build_chunked(elrt_ctx* ctx, int64_t E, double h, const double* h_el
             memcpy(&bits, ctx->h_pinned, sizeof(bits));
             float amax;
             memcpy(&amax, &bits, sizeof(amax));
-            f16 = amax >= kLuF16Max / 4096.f && amax <= kLuF16Max;
+            f16 = amax >= kLuF16Min && amax <= kLuF16Max;
         }
         if constexpr (sizeof(T) == 4) {
             if (tc) s = tc_lu_factor_solve(ctx, M, ld, estride, n, estat, side, ctx->d_flags + 2, tl.nrhs, f16);
