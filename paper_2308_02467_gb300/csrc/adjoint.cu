@@ -1,6 +1,6 @@
-// The last refinement step of a local build whose caller wants the FP32 operators alone (no statistics, no
+// The last refinement step of a TF32_IR build whose caller wants the FP32 operators alone (no statistics, no
 // status words, no A_i2u): the correction R A^{-1} r of the restricted operators by an adjoint product instead of a
-// re-solve of the whole system.
+// re-solve of the whole system.  (FP32_IR, whose products stay on the CUDA cores, keeps the re-solve.)
 //
 // With the residual r = -B^ - A X (float-float, residual.cu) the refined operators are in2out = R^o X +
 // R^o A^{-1} r and in2sol = R^m X + R^m A^{-1} r.  The discrete transport operator is reciprocal: with P the

@@ -1383,12 +1383,13 @@ elrt_status build_chunked(elrt_ctx* ctx, int64_t E, double h, const double* h_el
     const Tab& t = ctx->tab;
     const bool has_src = ex && ex->source;
     const bool ir = (mode != ELRT_LOCAL_FP64);
+    const bool tc = (mode == ELRT_LOCAL_TF32_IR);
     // one refinement step whose caller wants FP32 in2out / in2sol alone: the correction of the operators by
     // an adjoint product (adjoint.cu), with the isotropic unit sources as nm more right-hand sides.  A build
-    // with statistics, status words, a source or A_i2u needs the corrected solution itself, and FP64 operators
-    // the re-solve's last digits.
-    const bool adj = sizeof(T) == 4 && ir && steps == 1 && out_dtype == ELRT_F32 && !stats && !elem_status && !has_src && !(ex && ex->in2rad) &&
-                     residual_eo_fits(t) && adjoint_fits(t);
+    // with statistics, status words, a source or A_i2u needs the corrected solution itself, FP64 operators
+    // the re-solve's last digits; and FP32_IR computes on the CUDA cores, the correction too.
+    const bool adj = sizeof(T) == 4 && tc && steps == 1 && out_dtype == ELRT_F32 && !stats && !elem_status &&
+                     !has_src && !(ex && ex->in2rad) && residual_eo_fits(t) && adjoint_fits(t);
     Tab tl = t;  // the LU's right-hand sides: the -B^ columns, then the source column or the unit sources
     tl.nrhs = t.nin + (has_src ? 1 : 0) + (adj ? t.nm : 0);
     const int64_t ld = ((t.nu + tl.nrhs + 31) / 32) * 32;
@@ -1398,7 +1399,6 @@ elrt_status build_chunked(elrt_ctx* ctx, int64_t E, double h, const double* h_el
         for (int k = 0; k < t.N; ++k)
             for (int m = 0; m < t.n1; ++m) bmax = std::max(bmax, fabs(t.w[m] * t.sdn[F][k]));
     const bool want_res = ir || stats || elem_status;
-    const bool tc = (mode == ELRT_LOCAL_TF32_IR);
     const size_t side_per = tc ? tc_lu_side_floats(t, ld) * sizeof(float) : 0;
     // bytes per element: M, ipiv, status, maxres, the float-float or FP64 solution when refining /
     // measuring (the adjoint step: the residual and the angular sums), and the split operand buffers of the
