@@ -400,8 +400,8 @@ elrt_status elrt_solve_batch(elrt_ctx* const* ctxs, int32_t n_ctx, const elrt_fi
  *   restart      GMRES restart length of solve calls that pass restart = 0 (default 12).
  * elrt_autotune builds the local operators of `field` (device inputs as elrt_solve_field) with
  * every candidate (local_chunk in {0, 512, 1024, ...} below the field's element count, lu_pairs in
- * {1, 0} for ELRT_LOCAL_TF32_IR), timing each by CUDA events (one warm-up, mean of two), keeps the
- * fastest, then solves the skeleton system to rtol with restart lengths {8, 12, 16, 20, 30} and
+ * {1, 0} for ELRT_LOCAL_TF32_IR), with statistics, as elrt_solve_batch builds them, timing each by
+ * CUDA events (one warm-up, mean of two), keeps the fastest, then solves the skeleton system to rtol with restart lengths {8, 12, 16, 20, 30} and
  * keeps the fastest converged one.  It allocates its own temporary operators (the field's in2out
  * and in2sol in FP32), synchronises, and leaves the context unchanged on failure.  With the
  * environment variable ELRT_TUNE_CACHE naming a file, each result is appended there as one text

@@ -105,6 +105,9 @@ extern "C" elrt_status elrt_autotune(elrt_ctx* ctx, const elrt_field* fld, int32
     std::vector<int64_t> chunks{0};
     for (int64_t c = 512; c < E; c *= 2) chunks.push_back(c);
     std::vector<int> pairs{1};
+    // with statistics, as elrt_solve_batch and the fields of callers who read theirs build: without, a one-step
+    // TF32_IR build takes the adjoint product and no re-solve, half of the panel schedule's launches
+    elrt_local_stats ls{};
     if (mode == ELRT_LOCAL_TF32_IR) pairs.push_back(0);
     double best = 1e300;
     Tuning pick = ctx->tune;
@@ -114,7 +117,7 @@ extern "C" elrt_status elrt_autotune(elrt_ctx* ctx, const elrt_field* fld, int32
             ctx->tune.lu_pairs = pr;
             auto run = [&] {
                 return local_build(ctx, E, fld->h, nullptr, fld->kappa, fld->omega, mode, refine_steps, ELRT_F32, i2o,
-                                   i2m, nullptr, nullptr);
+                                   i2m, nullptr, &ls);
             };
             double ms = 0.0, ms2 = 0.0;
             s = time_events(ctx, run, &ms);  // (first run: warm-up and workspace growth)
@@ -138,7 +141,7 @@ extern "C" elrt_status elrt_autotune(elrt_ctx* ctx, const elrt_field* fld, int32
         r.local_ms_best = best;
         // operators of the chosen configuration, then the restart length
         s = local_build(ctx, E, fld->h, nullptr, fld->kappa, fld->omega, mode, refine_steps, ELRT_F32, i2o, i2m,
-                        nullptr, nullptr);
+                        nullptr, &ls);
     }
     if (!s) {
         best = 1e300;
