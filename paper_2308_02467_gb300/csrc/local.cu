@@ -241,9 +241,11 @@ __device__ __forceinline__ T tabs(T x) { return x < T(0) ? -x : x; }
 // searches (two barriers a column), the row swaps, the column solves.  The tile shapes below keep the rank
 // update's shared-memory traffic level with its FMAs (16 wavefronts per 64 FMAs a lane: a 16-byte load costs
 // four wavefronts even where lanes share addresses), a column's row swaps are one round of independent loads
-// (the panel's net permutation, net_swaps), and 16 warps share the panel.  Measured, 777 elements at p = 6,
-// N = 16, against 8 warps with the interchanges one by one: factorisation 39.3 -> 28.0 ms, re-solve
-// 15.3 -> 10.5 ms.
+// (the panel's net permutation, net_swaps), and 16 warps share the panel.  Small systems are bound by fetching
+// the unrolled code once: the interchanges are skipped where there are none and index in 32 bits.  Measured
+// against 8 warps with the interchanges one by one, FP32: 900 elements at p = 6, N = 16, factorisation 40.9 ->
+// 27.4 ms, re-solve 15.7 -> 10.3 ms; 16 elements at p = 2, N = 8, 129 -> 126 and 53 -> 47 us; at p = 1, N = 4 (one
+// panel) 30 -> 34 and 14 -> 15 us (37 and 18 with the interchanges fetched).
 
 // 16-byte vectors of T
 template <typename T> struct Vec;
@@ -367,7 +369,7 @@ __device__ void panel_forward(T* __restrict__ M, int64_t ld, int nu, int J, int 
                               T* Us, int c_begin, int c_end) {
     constexpr int CW = 32 * QN;
     constexpr int lds = NB + 1;
-    const int nd = sw.nd;
+    const int nd = sw.nd, ldi = (int)ld;  // (a matrix has fewer than 2^31 entries)
     for (int cs = c_begin; cs < c_end; cs += CW) {
         const int ncols = min(CW, c_end - cs);
         for (int tcol = threadIdx.x; tcol < CW; tcol += TH) {
@@ -375,13 +377,15 @@ __device__ void panel_forward(T* __restrict__ M, int64_t ld, int nu, int J, int 
                 T* col = M + (int64_t)J * ld + cs + tcol;
                 T x[NB], d[NB];
 #pragma unroll
-                for (int jj = 0; jj < NB; ++jj) x[jj] = (jj < jb) ? col[(int64_t)sw.occ[jj] * ld] : T(0);
+                for (int jj = 0; jj < NB; ++jj) x[jj] = (jj < jb) ? col[sw.occ[jj] * ldi] : T(0);
+                if (nd > 0) {  // (a panel with no rows below, or diagonal pivots, does not even fetch these)
 #pragma unroll
-                for (int q = 0; q < NB; ++q)
-                    if (q < nd) d[q] = col[(int64_t)sw.src[q] * ld];
+                    for (int q = 0; q < NB; ++q)
+                        if (q < nd) d[q] = col[sw.src[q] * ldi];
 #pragma unroll
-                for (int q = 0; q < NB; ++q)
-                    if (q < nd) col[(int64_t)sw.pos[q] * ld] = d[q];
+                    for (int q = 0; q < NB; ++q)
+                        if (q < nd) col[sw.pos[q] * ldi] = d[q];
+                }
 #pragma unroll
                 for (int jj = 1; jj < NB; ++jj) {
                     T s = x[jj];
@@ -391,7 +395,7 @@ __device__ void panel_forward(T* __restrict__ M, int64_t ld, int nu, int J, int 
                 }
 #pragma unroll
                 for (int jj = 0; jj < NB; ++jj) {
-                    if (jj < jb) col[(int64_t)jj * ld] = x[jj];
+                    if (jj < jb) col[jj * ldi] = x[jj];
                     Us[jj * CW + tcol] = (jj < jb) ? x[jj] : T(0);
                 }
             } else {
