@@ -1255,11 +1255,17 @@ double restrict_bytes(const Tab& t, size_t ss, size_t so, int64_t n) {
     return ((double)t.nu * t.nin * ss + (double)(t.nin + t.nm) * t.nin * so) * (double)n;
 }
 
-// Launches of the pivoted LU (shared with the allocation-free build).  512 threads once a panel has rows
-// for them, else 256 and two blocks per SM.  (Two blocks of 256 threads with 24-column panels at nu = 784,
-// so that one block's panel would overlap the other's updates, was slower: 46.9 against 43.4 ms for the
-// build of 777 elements.)
+// Launches of the pivoted LU (shared with the allocation-free build): TH threads per element.
+// While the panels of two blocks fit an SM (FP32 to nu = 620, FP64 to 722), two of 256 threads overlap one's
+// panel with the other's updates; beyond, one block shares the panel among 512.  Factorisation of 300 elements,
+// 256 against 512 threads, FP32: nu = 392 1.67 against 2.29 ms, 588 4.25 against 5.05, 648 6.90 against 5.91;
+// FP64: nu = 392 23.2 against 25.3 ms, 648 88.8 against 90.8.  A batch that gives an SM one element at most has
+// nothing to overlap: 512 threads above nu = 320 (100 elements, FP32: nu = 256 568 against 567 us, 320 838
+// against 806, 392 1207 against 1116; FP64: nu = 256 4.75 against 5.03 ms, 320 9.39 against 9.23, 432 17.8
+// against 17.2).  (Two blocks of 256 threads with 24-column panels at nu = 784 were slower: 46.9 against 43.4 ms
+// for the build of 777 elements.)
 constexpr int kLuWide = 320;
+constexpr size_t kLuTwo = 112 * 1024;  // dynamic shared memory of a block that leaves room for a second one
 template <typename T, int NB, int QN, int TH>
 cudaError_t lu_launch(const Tab& t, cudaStream_t st, T* M, int64_t ld, int64_t estride, int* ipiv, int* estat, int64_t n,
                       bool resolve) {
@@ -1276,10 +1282,11 @@ cudaError_t lu_launch(const Tab& t, cudaStream_t st, T* M, int64_t ld, int64_t e
     return e == cudaSuccess ? cudaGetLastError() : e;
 }
 template <typename T, int NB, int QN>
-cudaError_t lu_run(const Tab& t, cudaStream_t st, T* M, int64_t ld, int64_t estride, int* ipiv, int* estat, int64_t n,
-                   bool resolve) {
-    return t.nu > kLuWide ? lu_launch<T, NB, QN, 512>(t, st, M, ld, estride, ipiv, estat, n, resolve)
-                          : lu_launch<T, NB, QN, 256>(t, st, M, ld, estride, ipiv, estat, n, resolve);
+cudaError_t lu_run(const Tab& t, int sms, cudaStream_t st, T* M, int64_t ld, int64_t estride, int* ipiv, int* estat,
+                   int64_t n, bool resolve) {
+    const bool wide = n <= sms ? t.nu > kLuWide : lu_smem_bytes<T, NB, QN>(t.nu) > kLuTwo;
+    return wide ? lu_launch<T, NB, QN, 512>(t, st, M, ld, estride, ipiv, estat, n, resolve)
+                : lu_launch<T, NB, QN, 256>(t, st, M, ld, estride, ipiv, estat, n, resolve);
 }
 
 // t: the context's table with nrhs set to the right-hand-side columns of this build
@@ -1293,7 +1300,7 @@ elrt_status run_lu(elrt_ctx* ctx, const Tab& t, T* M, int64_t ld, int64_t estrid
                  resolve ? (double)n * (sizeof(T) * (nu * nu + 2.0 * nu * nin) + 4.0 * nu)
                          : (double)n * (2.0 * sizeof(T) * nu * (nu + nin) + 4.0 * nu),
                  (double)n * ((resolve ? 0.0 : 2.0 / 3.0 * nu * nu * nu) + 2.0 * nu * nu * nin));
-    return cuda_check(ctx, lu_run<T, NB, QN>(t, ctx->stream, M, ld, estride, ipiv, estatus, n, resolve), "lu launch");
+    return cuda_check(ctx, lu_run<T, NB, QN>(t, ctx->sms, ctx->stream, M, ld, estride, ipiv, estatus, n, resolve), "lu launch");
 }
 
 template <typename T>
@@ -1653,6 +1660,7 @@ namespace {
 constexpr size_t kStaticBytes = (size_t)ELRT_STATIC_SCRATCH_MIB << 20;
 constexpr size_t kStaticHead = 256;  // input-validation flag
 constexpr int kStaticMaxDevices = 64;
+constexpr int kStaticSms = 152;  // SMs of a GB300
 void* g_static_addr[kStaticMaxDevices];
 std::once_flag g_static_once[kStaticMaxDevices];
 cudaError_t g_static_err[kStaticMaxDevices];
@@ -1711,13 +1719,13 @@ elrt_status static_build(const Tab& t, cudaStream_t sm, unsigned char* scratch, 
         const double* om = omega + e0;
         if (cudaMemsetAsync(estat, 0, n * sizeof(int), sm) != cudaSuccess) return ELRT_ECUDA;
         k_assemble<T><<<dim3((unsigned)n, t.N), kThreads, 0, sm>>>(t, h, he, ka, om, M, ld, estride, nullptr, 0, flags, 0);
-        if (lu_run<T, NB, QN>(t, sm, M, ld, estride, ipiv, estat, n, false)) return ELRT_ECUDA;
+        if (lu_run<T, NB, QN>(t, kStaticSms, sm, M, ld, estride, ipiv, estat, n, false)) return ELRT_ECUDA;
         void* o_i2o = (unsigned char*)in2out + (size_t)e0 * t.nin * t.nin * osz;
         void* o_i2m = (unsigned char*)in2sol + (size_t)e0 * t.nm * t.nin * osz;
         if (ir) {
             k_residual<T><<<(unsigned)n, kThreads, res_smem, sm>>>(t, h, he, ka, om, M, ld, estride, X64, 0, cwr, maxres, n);
             for (int it = 0; it < steps; ++it) {
-                if (lu_run<T, NB, QN>(t, sm, M, ld, estride, ipiv, estat, n, true)) return ELRT_ECUDA;
+                if (lu_run<T, NB, QN>(t, kStaticSms, sm, M, ld, estride, ipiv, estat, n, true)) return ELRT_ECUDA;
                 k_residual<T><<<(unsigned)n, kThreads, res_smem, sm>>>(t, h, he, ka, om, M, ld, estride, X64, 1, cwr,
                                                                       maxres, n);
             }
@@ -1735,7 +1743,7 @@ elrt_status static_build(const Tab& t, cudaStream_t sm, unsigned char* scratch, 
                 k_restrict<T, double><<<(unsigned)n, kThreads, 0, sm>>>(t, M, ld, estride, t.nu, (double*)o_i2o,
                                                                        (double*)o_i2m, estat, n);
         }
-        k_static_status<<<(unsigned)std::min<int64_t>(152, (n + 255) / 256), 256, 0, sm>>>(estat, n, flags);
+        k_static_status<<<(unsigned)std::min<int64_t>(kStaticSms, (n + 255) / 256), 256, 0, sm>>>(estat, n, flags);
         if (cudaGetLastError() != cudaSuccess) return ELRT_ECUDA;
     }
     int bad[2] = {0, 0};
