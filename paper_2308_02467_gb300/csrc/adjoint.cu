@@ -42,7 +42,15 @@ namespace {
 constexpr int kAdjWarps = 15;                      // operand warps
 constexpr int kAdjThreads = 32 * (kAdjWarps + 1);  // and the MMA warp; all sixteen run the epilogue
 constexpr int kAdjK = 32;                          // rows of the sum per stage: 128 bytes of FP32
-constexpr int kAdjSmem = 220 * 1024;
+// tables of the columns (xrow, orow, scale, us below); with the barriers they are the kernel's static shared
+// memory, which the stages' alignment rounds up to 1 KB (ptxas: 10,240 bytes).  The rest of the 227 KB a block
+// can have holds the stages
+constexpr int kAdjCols = 4 * ELRT_MAX_N1 * ELRT_MAX_ANG / 2;
+constexpr int kAdjStatic = (kAdjCols * (int)(sizeof(int) + sizeof(short) + 2 * sizeof(float)) + 64 + 1023) / 1024 * 1024;
+constexpr int kAdjSmem = 227 * 1024 - kAdjStatic;
+// dynamic shared memory of a launch with that many stages and nc columns (1024: the stages' alignment)
+constexpr int adj_smem(int stages, int nc) { return stages * 2 * 128 * (128 + nc) + 1024; }
+static_assert(adj_smem(1, 512) <= kAdjSmem, "one stage of the widest product fits");
 
 struct AdjArgs {
     const float* M;        // [E][nu][ld], solution columns from nu: X, then Z
@@ -82,10 +90,10 @@ __global__ void __launch_bounds__(kAdjThreads, 1)
     __shared__ uint64_t full[2], empty[2], acc_full;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_s;
-    __shared__ int xrow[4 * ELRT_MAX_N1 * ELRT_MAX_ANG / 2];          // row of X at the outflow value of column c
-    __shared__ short orow[4 * ELRT_MAX_N1 * ELRT_MAX_ANG / 2];        // its row of in2out
-    __shared__ float scale[4 * ELRT_MAX_N1 * ELRT_MAX_ANG / 2];       // 1 / the column's (scaled) entry of -B^
-    __shared__ float us[4 * ELRT_MAX_N1 * ELRT_MAX_ANG / 2];          // 1 / the column's power-of-two scale
+    __shared__ int xrow[kAdjCols];    // row of X at the outflow value of column c
+    __shared__ short orow[kAdjCols];  // its row of in2out
+    __shared__ float scale[kAdjCols]; // 1 / the column's (scaled) entry of -B^
+    __shared__ float us[kAdjCols];    // 1 / the column's power-of-two scale
     volatile int* abort = &abort_s;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t e = blockIdx.x / g.jtiles;
@@ -313,10 +321,9 @@ elrt_status adjoint_correct(elrt_ctx* ctx, const float* M, int64_t ld, int64_t e
     g.jtiles = (t.nin + 127) / 128;
     g.jw = ((t.nin + g.jtiles - 1) / g.jtiles + 15) / 16 * 16;
     g.nc = adj_nc(t);
-    const int stage = 2 * 128 * (128 + g.nc);
-    g.stages = 2 * stage <= kAdjSmem - 1024 ? 2 : 1;
+    g.stages = adj_smem(2, g.nc) <= kAdjSmem ? 2 : 1;
     g.err = err;
-    const int smem = g.stages * stage + 1024;
+    const int smem = adj_smem(g.stages, g.nc);
     cudaError_t e = allow_smem(k_adjoint);
     if (e != cudaSuccess) return cuda_check(ctx, e, "smem attribute");
     ProfScope ps(ctx, "adjoint", 1,
