@@ -33,20 +33,25 @@ WORKLOAD = workload_name(64)
 # bounds each: "hbm" (algorithmic bytes / time against the measured copy bandwidth) or "alu" with
 # the pipe whose issue rate limits it.  The float-float residual counts one useful flop per
 # multiply or add of the structured operator; one float-float multiply-add takes 12 FP32 issue
-# slots (1 MUL, 3 FMA, 6 in TwoSum, 2 ADD), so its ALU peak is the FP32 rate x 2 / 12.
+# slots (1 MUL, 3 FMA, 6 in TwoSum, 2 ADD), so its ALU peak is the FP32 rate x 2 / 12.  The kernels
+# of the common element shapes split every sum into an even and an odd part and execute about half
+# of the counted multiply-adds, so the pipe's own share is about half of their fraction.
 # The trailing update of the tensor-core LU is a dense contraction that also streams its trailing
 # tiles through HBM: "roof" takes whichever floor binds, the bytes at the copy bandwidth or the
 # issued flops (each product three times, hi*hi + lo*hi + hi*lo) at the TF32 tensor peak, and
 # reports the achieved fraction of that roof (the other fraction beside it).  The factorisation's
 # updates and the refinement re-solves' forward sweeps form their products in 3xFP16, at twice the
 # TF32 rate, so the tensor fraction counted at the TF32 rate is an upper bound on the tensor pipe's
-# share.
+# share.  The adjoint product of a one-step build is such a contraction too, in 3xTF32.
 KERNEL_BOUND = {
     "assemble": ("hbm", None), "lu_factor_solve": ("alu", "fp32"), "lu_resolve": ("hbm", None),
     "lu_tc_diag": ("alu", "fp32"), "lu_tc_rowcol": ("hbm", None), "lu_tc_update": ("roof", "tf32x3"),
     "residual": ("alu", "ff"), "restrict": ("hbm", None), "gemv": ("hbm", None), "krylov": ("hbm", None),
-    "sweep": ("hbm", None),
+    "sweep": ("hbm", None), "adjoint": ("roof", "tf32x3"),
 }
+# every group the profiled pass reads ("status", a flag reduction, has no row of its own)
+PROFILE_GROUPS = ("assemble", "lu_factor_solve", "lu_resolve", "lu_tc_diag", "lu_tc_rowcol", "lu_tc_update", "residual",
+                  "adjoint", "restrict", "status", "gemv", "krylov", "sweep")
 TENSOR_PASSES = {"tf32x3": 3}
 # Nominal dense tensor rates of GB300 (PFLOP/s): TF32 1.1, BF16 2.25.  A TF32 peak is the measured
 # BF16 peak times their ratio.
@@ -59,12 +64,10 @@ def tensor_peak_tflops(peaks):
     return peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"]) * TF32_PER_BF16
 # DRAM bytes (read + write) per element and step of each kernel group, from one ncu capture of
 # the 32 x 32 slab (1024 elements, one local-build chunk; summary kept under profiles/); a group
-# missing here has no capture of its current kernel (the trailing update and the panel solves
-# changed after it: FP16 forward re-solves, the grouped last panel of the backward sweeps).  Scaled
+# missing here has no capture of its current kernel (the trailing update, the panel solves and the
+# residual changed after it, the assembly writes more columns in a one-step build).  Scaled
 # to a launch of the benchmark by elements / launches.
-DRAM_BYTES_PER_ELEMENT_STEP = {
-    "lu_tc_diag": 3.275e5, "residual": 3.704e6, "assemble": 3.174e6, "restrict": 2.905e6,
-}
+DRAM_BYTES_PER_ELEMENT_STEP = {"lu_tc_diag": 3.275e5, "restrict": 2.905e6}
 
 
 def max_over_ranks(x, device):
@@ -917,10 +920,8 @@ def run_ours(args, rank, world, local_rank):
     ev3.record(stream)
     torch.cuda.synchronize()
     ms_profiled = ev2.elapsed_time(ev3) / args.steps
-    names = ("assemble", "lu_factor_solve", "lu_resolve", "lu_tc_diag", "lu_tc_rowcol", "lu_tc_update", "residual",
-             "adjoint", "restrict", "status", "gemv", "krylov", "sweep")
-    prof = {k: ctx.elrt_profile_get(k) for k in names}
-    work = {k: ctx.elrt_profile_work(k) for k in names}
+    prof = {k: ctx.elrt_profile_get(k) for k in PROFILE_GROUPS}
+    work = {k: ctx.elrt_profile_work(k) for k in PROFILE_GROUPS}
     ctx.elrt_profile_enable(False)
     ms = max_over_ranks(ms, "cuda")
 
