@@ -63,7 +63,13 @@ typedef enum {
  * bits, error-free TwoSum / FMA TwoProduct) with the running solution X also kept in float-float;
  * no FP64 instruction runs per matrix entry.  Measured: one sweep takes the FP32-level solution to a
  * maximum relative residual of ~2e-12 on the benchmark slab; two sweeps stay below 1e-12 on every
- * tested element. */
+ * tested element.
+ * One exception: a TF32_IR build with refine_steps = 1, out_dtype ELRT_F32 and neither statistics, status
+ * words, a source nor in2rad corrects the operators instead of X, by one product (3xTF32 on the tensor
+ * cores) of the residual with the solutions of the reversed directions, for even p <= 8 with 8, 12 or 16
+ * cells and p = 6 with 28.  Its operators differ from the corrected solution's by up to ~3e-11 on the
+ * benchmark slab (p = 8: 6e-11), below the rounding to FP32 of all entries above 1e-3; asking for
+ * statistics or status words selects the re-solve, and they describe that build. */
 typedef enum {
     ELRT_LOCAL_FP64 = 0,     /* FP64 LU with partial pivoting on the CUDA cores (no refinement) */
     ELRT_LOCAL_FP32_IR = 1,  /* FP32 LU with partial pivoting on the CUDA cores, then float-float refinement */

@@ -16,9 +16,12 @@
 // residual of that size, so the refined operators are as accurate as with a re-solve -- provided the columns
 // of X are accurate relative to their own size: the assembly scales each -B^ column by a power of two so that
 // its entry lies in [0.5, 1), and the epilogue takes the scales out again (without, the 3xFP16 factorisation
-// left a thick element's grazing columns thirteen times less accurate than the re-solve).  The product sums 784
-// terms in tensor memory, whose additions truncate: ~2e-11 of error in an operator entry where a re-solve
-// leaves ~3e-12, both far below the FP32 rounding of the result (6e-8); FP64 operators keep the re-solve.
+// left a thick element's grazing columns thirteen times less accurate than the re-solve).  Before the rounding
+// to FP32 it leaves more than a re-solve does: on 256 elements of the slab (p = 6, N = 16) at most 2.7e-11 in in2out
+// and 6.8e-12 in in2sol where the re-solve leaves 6.4e-12 and 4.2e-13, since its second factor has the 3xFP16
+// factorisation's backward sweep (with 3xTF32 factors 2.4e-12 and 3.3e-13 against 1.4e-12 and 6.0e-14).  The rounded
+// operators' largest and mean-square errors are the same to three digits, 5.9e-8 and 1.1e-9; entries below
+// ~1e-3 carry the difference.  FP64 operators keep the re-solve.
 //
 // k_adjoint: one CTA per (element, tile of up to 128 of the n_in columns of r): D[j][c] = sum_rows r[row][j]
 // XZ[reversed row][c] in 3xTF32 on the tensor cores (FP32 values are their own high part; the full FP32 range,
@@ -27,10 +30,11 @@
 // columns a lane), transpose in registers and write K-major, 128-byte-swizzled tiles of 32 rows of the sum,
 // eight lanes on one row's eight chunks (no bank conflicts); one thread of a sixteenth warp issues the MMAs.
 // Bound by the latency of its loads (about 2.4 MB per element in two column tiles, the second tile's mostly
-// from L2; DRAM 25 % and the tensor pipe 28 % busy): 16 warps and two stages of 106 KB are what one SM holds.  The epilogue reads X at the outflow rows, adds the correction
-// and rounds once.  Measured, builds with one refinement step: 4096 elements at p = 6, N = 16, 61.9 -> 51.6 ms
-// (the re-solve and the float-float restriction gone, k_adjoint 4.4 ms, the 49 columns 2 ms), 50.8 ms with its
-// loads as below; nine elements 1.92 -> 1.28 ms (141 -> 90 launches).
+// from L2; DRAM 25 % and the tensor pipe 28 % busy): 16 warps and two stages of 106 KB are what one SM holds.
+// The epilogue reads X at the outflow rows, adds the correction and rounds once.  Measured, builds with one
+// refinement step: 4096 elements at p = 6, N = 16, 61.9 -> 51.6 ms (the re-solve and the float-float restriction
+// gone, k_adjoint 4.4 ms, the 49 columns 2 ms), 50.8 ms with its loads as below; nine elements 1.92 -> 1.28 ms
+// (141 -> 90 launches).
 #include <algorithm>
 
 #include "elrt_internal.h"

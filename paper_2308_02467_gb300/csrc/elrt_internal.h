@@ -155,6 +155,7 @@ elrt_status residual_eo(elrt_ctx* ctx, double h, const double* h_elem, const dou
 
 // ---- last refinement step by an adjoint product (adjoint.cu)
 bool adjoint_fits(const Tab& t);
+constexpr int kAdjErr = 4096 | 8192;  // its codes in the LU's error flag: an epilogue or an MMA wait gave up
 elrt_status adjoint_correct(elrt_ctx* ctx, const float* M, int64_t ld, int64_t estride, const float* R, const void* sum,
                             float* in2out, float* in2sol, int* err, int64_t n);
 

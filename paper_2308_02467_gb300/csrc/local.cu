@@ -1338,8 +1338,7 @@ elrt_status launch_residual_ff(elrt_ctx* ctx, double h, const double* h_elem, co
     const int cwr = residual_ff_cwr(t, sizeof(XS));
     if (cwr < 2) return ctx_fail(ctx, ELRT_EINVAL, "float-float residual: element too large for two staged columns");
     const size_t smem = residual_ff_smem(t, cwr, sizeof(XS));
-    cudaError_t e =
-        allow_smem(k_residual_ff<XS>);
+    cudaError_t e = allow_smem(k_residual_ff<XS>);
     if (e != cudaSuccess) return cuda_check(ctx, e, "smem attribute");
     // a batch too small to fill the GPU spreads each element's column chunks over several blocks
     const int nchunk = (t.nin + cwr - 1) / cwr;
@@ -1620,7 +1619,9 @@ elrt_status build_chunked(elrt_ctx* ctx, int64_t E, double h, const double* h_el
     prof_flush(ctx);
     const int* hf = (const int*)ctx->h_pinned;
     if (hf[0]) return ctx_fail(ctx, ELRT_EINVAL, "negative/non-finite kappa or h, or omega outside [0,1]");
-    if (hf[2]) return ctx_fail(ctx, ELRT_ETIMEOUT, "a tensor-core LU wait timed out (code " + std::to_string(hf[2]) + ")");
+    if (hf[2])
+        return ctx_fail(ctx, ELRT_ETIMEOUT, std::string("a wait of the ") + (hf[2] & ~kAdjErr ? "tensor-core LU" : "adjoint product") +
+                                                " timed out (code " + std::to_string(hf[2]) + ")");
     if (stats) {
         stats->refine_steps = ir ? steps : 0;
         stats->n_flagged = hf[1];
@@ -1708,8 +1709,7 @@ elrt_status static_build(const Tab& t, cudaStream_t sm, unsigned char* scratch, 
     double* maxres = X64 + (ir ? (size_t)chunk * t.nu * t.nin : 0);
     int* ipiv = (int*)(maxres + chunk);
     int* estat = ipiv + (size_t)chunk * t.nu;
-    if (allow_smem(k_residual<T>))
-        return ELRT_ECUDA;
+    if (allow_smem(k_residual<T>)) return ELRT_ECUDA;
     if (cudaMemsetAsync(flags, 0, 2 * sizeof(int), sm) != cudaSuccess) return ELRT_ECUDA;
     const size_t osz = out_dtype == ELRT_F32 ? sizeof(float) : sizeof(double);
     for (int64_t e0 = 0; e0 < E; e0 += chunk) {

@@ -904,8 +904,8 @@ bool map3_16(CUtensorMap* m, const float* p, int64_t rows, int64_t E, int box_ro
 }
 
 // the matrix of every element seen as [E][rows][cols] (row pitch ld), box 32 columns x 128 rows x 1
-// element, 128-byte swizzle: with rows = nu, cols = ld the C tiles of the loads; with rows = r_end,
-// cols = c_end the stores of an update (whatever lies outside is clipped)
+// element, 128-byte swizzle: rows = r_end and cols = c_end of an update, whose C tiles are loaded and stored
+// through it (what lies outside is neither read nor written)
 bool mapM(CUtensorMap* m, const float* M, int64_t rows, int64_t cols, int64_t ld, int64_t estride, int64_t E) {
     cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)E};
     cuuint64_t strides[2] = {(cuuint64_t)ld * 4, (cuuint64_t)estride * 4};
@@ -924,8 +924,8 @@ struct TcMaps {
 
 // Trailing update C -= L U over rows [r0, r_end) and columns [c0, c_end) of every element, with
 // L = M[rows, J .. J+k) and U^T from the side buffer at K offset koff: rank k = jb <= 64 (one panel,
-// kernel NK = 64) or 64 < k <= 128 (a pair of panels, the second possibly partial, NK = 128, koff 0;
-// the strip is zero beyond jb).  Algorithmic bytes: C read and written, the FP32 L strip (R x k) and
+// kernel NK = 64), 64 < k <= 128 (a pair of panels, the second possibly partial, NK = 128) or, in 3xFP16 alone,
+// k <= 256 (four panels, NK = 256, koff 0); the strip is zero beyond jb.  Algorithmic bytes: C read and written, the FP32 L strip (R x k) and
 // U^T tile (C x k); useful flops 2 R C k.
 template <int NK>
 elrt_status update(elrt_ctx* ctx, const TcMaps& mp, float* M, int64_t ld, int64_t estride, int64_t E, int J, int jb,

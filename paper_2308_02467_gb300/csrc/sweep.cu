@@ -637,9 +637,9 @@ size_t sweep_words_bytes(const Tab& t, int64_t E) { return (size_t)4 * E * (t.ni
 bool sweep_needs_order(const Tab& t, int nx, int nz, int sms) { return line_stages(t, nx, nz, 4, sms) == 0; }
 
 // z = M u on the stream, with the operator A (FP16 or FP32, [E][nin][nin], 16-byte aligned);
-// order: device [4 E] from sweep_orders (not read where sweep_needs_order says no); zw: device scratch of sweep_words_bytes; flags: device ints
-// (err, abort), cleared here (err stays set after a timed-out wait); z is zeroed first, so a skipped
-// application leaves 0.
+// order: device [4 E] from sweep_orders (not read where sweep_needs_order says no); zw: device scratch of
+// sweep_words_bytes; flags: device ints (err, abort), cleared here (err stays set after a timed-out wait); z is
+// zeroed first, so a skipped application leaves 0.
 elrt_status sweep_apply(elrt_ctx* ctx, int nx, int nz, const void* A, int a_bytes, const float* u, float* z,
                         const int* order, void* zw, int* flags, const int* done, const int* nsteps) {
     const Tab& t = ctx->tab;
