@@ -382,8 +382,10 @@ elrt_status launch_mode(const Args& a, int mode) {
 
 }  // namespace
 
-// Shapes with a kernel here: p in {2, 4, 6, 8} with 8, 12 or 16 angular cells, and p = 6 with 28.  Others
-// take the general kernel of local.cu.
+// Shapes with a kernel here: p in {2, 4, 6, 8} with 8, 12 or 16 angular cells, and p = 6 with 28, those of the
+// workloads.  Each is three compiled instances with its sums unrolled, which is what bounds the list; the split
+// itself needs an odd number of nodes per line and an even number of cells.  Others take the general kernel of
+// local.cu (and builds of theirs the re-solve).
 bool residual_eo_fits(const Tab& t) {
     const bool n = t.N == 8 || t.N == 12 || t.N == 16;
     return (n && (t.n1 == 3 || t.n1 == 5 || t.n1 == 7 || t.n1 == 9)) || (t.n1 == 7 && t.N == 28);
